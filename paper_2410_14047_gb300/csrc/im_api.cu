@@ -298,6 +298,13 @@ struct im_sketch {
     // a selection in flight: phases and rebuilds queue without host reads;
     // their error word is read once at the end
     bool defer = false;
+    // the set of per-level counters, formats and barrier words the current phase
+    // uses, and each set's state: a persistent phase zeroes the other set when
+    // the phase before it ran there
+    int pset = 0;
+    int fmt0 = 0;  // format of the current phase's level-0 queue
+    enum SetState { kSetDirty, kSetZeroed, kSetUsed };
+    SetState set_state[2] = {kSetDirty, kSetDirty};
     bool pull_safe = false;  // the pull queue holds every out-bucket (it cannot overflow)
     DBuf out_seed, out_S, out_est;
     DBuf gsum;  // lazy-pick group records
@@ -682,6 +689,8 @@ extern "C" im_status im_graph_info(const im_graph* g, int32_t* n, int64_t* m) {
 // ---------------------------------------------------------------------------
 // sketches
 // ---------------------------------------------------------------------------
+constexpr size_t kSetLevels = kMaxLevels + 2;  // per-level counters of one set
+
 // Device buffers of a sketch of J simulations over n vertices, with their
 // sizes; sketch_alloc allocates exactly this list and query_bytes sums it.
 using BufPlan = std::vector<std::pair<DBuf*, size_t>>;
@@ -693,8 +702,9 @@ static void sketch_plan(im_sketch* sk, int32_t n, int64_t m_edges, int32_t J, Bu
     A(sk->X, (size_t)J * 4);
     A(sk->salt, (size_t)J * 4);
     A(sk->tab, (size_t)kTabSize * 2);
-    A(sk->ctr, (size_t)(kMaxLevels + 2) * 16);
-    A(sk->claim, (size_t)(kMaxLevels + 2) * 4);
+    // two sets of the per-level counters, formats and barrier words: phases alternate
+    A(sk->ctr, 2 * kSetLevels * 16);
+    A(sk->claim, 2 * kSetLevels * 4);
     for (int i = 0; i < 3; ++i) A(sk->chg[i], (size_t)n * ((J + 31) / 32) * 4);
     A(sk->gen, (size_t)n * 4);
     A(sk->seed_bits, (((size_t)n + 31) / 32) * 4);
@@ -704,9 +714,9 @@ static void sketch_plan(im_sketch* sk, int32_t n, int64_t m_edges, int32_t J, Bu
     A(sk->ticket, 4);
     A(sk->stats, (size_t)kStCount * 8);
     A(sk->err, 4);
-    A(sk->bar, 256);  // barrier words: arrivals, abort, levels; generation from byte 128
+    A(sk->bar, 2 * kBarWords * 4);
     A(sk->level_ns, (size_t)(kMaxLevels + 2) * 8);
-    A(sk->fmt, (size_t)(kMaxLevels + 2));
+    A(sk->fmt, 2 * kSetLevels);
     // incremental rebuilds: newly visited and affected register bits, the
     // affected vertices
     A(sk->nv, (size_t)n * ((J + 31) / 32) * 4);
@@ -931,26 +941,38 @@ static im_status check_err(im_sketch* sk) {
     return IM_OK;
 }
 
-// Start of a propagation or cover phase: level counters and work counters
-// back to zero.  A phase that completes leaves its change masks zero (the
-// last level's bits are cleared by the phase itself); after a new sketch or a
+// The current set's counters, work counters, formats and barrier words.
+static ulonglong2* set_ctr(const im_sketch* sk, int set) { return sk->ctr.as<ulonglong2>() + set * kSetLevels; }
+static unsigned int* set_claim(const im_sketch* sk, int set) { return sk->claim.as<unsigned int>() + set * kSetLevels; }
+static uint8_t* set_fmt(const im_sketch* sk, int set) { return sk->fmt.as<uint8_t>() + set * kSetLevels; }
+static unsigned int* set_bar(const im_sketch* sk, int set) { return sk->bar.as<unsigned int>() + set * kBarWords; }
+static ulonglong2* cur_ctr(const im_sketch* sk) { return set_ctr(sk, sk->pset); }
+
+// Start of a propagation or cover phase: the other set of level counters, work
+// counters and barrier words, zeroed unless the last persistent phase did so
+// already.  A phase that completes leaves its change masks zero (the last
+// level's bits are cleared by the phase itself); after a new sketch or a
 // failed phase they are cleared here.
 static im_status phase_begin(im_sketch* sk, int mode, int fmt0 = -1) {
     im_ctx* c = sk->ctx;
     auto st = c->stream;
-    CK(c, cudaMemsetAsync(sk->ctr.p, 0, sk->ctr.bytes, st));
+    sk->pset ^= 1;
+    const int s = sk->pset;
+    if (sk->set_state[s] != im_sketch::kSetZeroed) {
+        CK(c, cudaMemsetAsync(set_ctr(sk, s), 0, kSetLevels * 16, st));
+        CK(c, cudaMemsetAsync(set_claim(sk, s), 0, kSetLevels * 4, st));
+        CK(c, cudaMemsetAsync(set_bar(sk, s), 0, kBarWords * 4, st));
+        sk->set_state[s] = im_sketch::kSetZeroed;
+    }
     // the level-0 queue: bucket entries (fmt0 = 1, or by default for a cover
     // in bucket mode: the seed kernel writes them), vertex entries otherwise
-    if (fmt0 < 0) fmt0 = (mode == kCover && sk->buckets) ? 1 : 0;
-    CK(c, cudaMemsetAsync(sk->fmt.p, fmt0, 1, st));
-    CK(c, cudaMemsetAsync(sk->claim.p, 0, sk->claim.bytes, st));
+    sk->fmt0 = fmt0 >= 0 ? fmt0 : ((mode == kCover && sk->buckets) ? 1 : 0);
     if (sk->chg_dirty) {
         for (int i = 0; i < 3; ++i) CK(c, cudaMemsetAsync(sk->chg[i].p, 0, sk->chg[i].bytes, st));
         for (int i = 0; i < 3; ++i)
             if (sk->chg_cov[i].p) CK(c, cudaMemsetAsync(sk->chg_cov[i].p, 0, sk->chg_cov[i].bytes, st));
         sk->chg_dirty = false;
     }
-    CK(c, cudaMemsetAsync(sk->bar.p, 0, sk->bar.bytes, st));
     return IM_OK;
 }
 
@@ -969,21 +991,24 @@ static im_status run_phase_persistent(im_sketch* sk, int mode, bool all_first, i
         p.qh[i] = sk->qh[i].as<QEntry>();
         p.chg[i] = chg_buf(sk, mode, i).as<uint32_t>();
     }
-    p.ctr = sk->ctr.as<ulonglong2>();
-    p.claim = sk->claim.as<unsigned int>();
+    const int s = sk->pset, o = s ^ 1;
+    p.ctr = set_ctr(sk, s);
+    p.claim = set_claim(sk, s);
     p.all_first = all_first ? 1 : 0;
     p.max_levels = c->max_levels;
     p.gen_base = sk->gen_counter + 1;
-    unsigned int* bar = sk->bar.as<unsigned int>();
-    // the generation word (polled by the waiting blocks) on its own 128-byte
-    // line, away from the arrival counter
-    p.bar_arrive = bar;
-    p.abort_flag = bar + 2;
-    p.levels_out = reinterpret_cast<int*>(bar + 3);
-    p.bar_gen = bar + 32;
+    p.bar = set_bar(sk, s);
     p.limit_ns = c->barrier_limit_ns;
     p.level_ns = c->trace ? sk->level_ns.as<unsigned long long>() : nullptr;
-    p.fmt = sk->fmt.as<uint8_t>();
+    p.fmt = set_fmt(sk, s);
+    p.fmt0 = sk->fmt0;
+    if (sk->set_state[o] == im_sketch::kSetUsed) {
+        p.ctr_old = set_ctr(sk, o);
+        p.claim_old = set_claim(sk, o);
+        p.bar_old = set_bar(sk, o);
+        sk->set_state[o] = im_sketch::kSetZeroed;
+    }
+    sk->set_state[s] = im_sketch::kSetUsed;
     CK(c, timed(c, mode == kPush ? kTPush : kTCover,
                 [&] { return launch_phase(sk->kind, mode, sk->dev, p, grid, st); }));
     // stamps gen_base .. gen_base + max_levels are this phase's
@@ -996,16 +1021,15 @@ static im_status run_phase_persistent(im_sketch* sk, int mode, bool all_first, i
         sk->chg_dirty = false;  // a failed phase fails the whole selection
         return IM_OK;
     }
-    CK(c, cudaMemcpyAsync(c->pinned, bar, 16, cudaMemcpyDeviceToHost, st));
+    CK(c, cudaMemcpyAsync(c->pinned, p.bar + kBarLevels, 4, cudaMemcpyDeviceToHost, st));
     CK(c, sync_collect(c));
-    const unsigned int* hb = reinterpret_cast<const unsigned int*>(c->pinned);
-    const int levels = (int)hb[3];
+    const int levels = *reinterpret_cast<const int*>(c->pinned);
     sk->chg_dirty = true;
     if (c->trace && levels > 0 && levels < p.max_levels) {
         // per-level records from the in-kernel clock (one launch for all levels)
         std::vector<ulonglong2> h((size_t)levels);
         std::vector<unsigned long long> ns((size_t)levels + 1);
-        CK(c, cudaMemcpyAsync(h.data(), sk->ctr.p, (size_t)levels * 16, cudaMemcpyDeviceToHost, st));
+        CK(c, cudaMemcpyAsync(h.data(), p.ctr, (size_t)levels * 16, cudaMemcpyDeviceToHost, st));
         CK(c, cudaMemcpyAsync(ns.data(), sk->level_ns.p, ((size_t)levels + 1) * 8, cudaMemcpyDeviceToHost, st));
         CK(c, sync_collect(c));
         for (int l = 0; l < levels; ++l) {
@@ -1038,8 +1062,12 @@ static im_status run_levels(im_sketch* sk, int mode, bool all_first) {
         const int pgrid = std::min(phase_grid(), 64 * 32);
         if (pgrid > 0) return run_phase_persistent(sk, mode, all_first, pgrid);
     }
-    ulonglong2* ctr = sk->ctr.as<ulonglong2>();
-    unsigned int* claim = sk->claim.as<unsigned int>();
+    // per-level launches: the counters stay dirty, the level-0 format is in memory
+    sk->set_state[sk->pset] = im_sketch::kSetDirty;
+    ulonglong2* ctr = cur_ctr(sk);
+    unsigned int* claim = set_claim(sk, sk->pset);
+    uint8_t* fmt = set_fmt(sk, sk->pset);
+    CK(c, cudaMemsetAsync(fmt, sk->fmt0, 1, st));
     LevelArgs a = level_args(sk);
     set_lcm(a, sk, mode);
     const int grid = c->tuning.grid_blocks > 0 ? c->tuning.grid_blocks : level_grid();
@@ -1071,9 +1099,9 @@ static im_status run_levels(im_sketch* sk, int mode, bool all_first) {
         a.all_changed = (t == 0 && all_first) ? 1 : 0;
         a.claim = claim + t;
         a.gen_next = ++sk->gen_counter;
-        a.fmt_in = sk->fmt.as<uint8_t>() + t;
-        a.fmt_out = sk->fmt.as<uint8_t>() + t + 1;
-        a.fmt_prev = t >= 1 ? sk->fmt.as<uint8_t>() + t - 1 : nullptr;
+        a.fmt_in = fmt + t;
+        a.fmt_out = fmt + t + 1;
+        a.fmt_prev = t >= 1 ? fmt + t - 1 : nullptr;
         CK(c, timed(c, mode == kPush ? kTPush : kTCover,
                     [&] { return launch_level(sk->kind, mode, sk->dev, a, grid, st); }));
         ++t;
@@ -1106,9 +1134,9 @@ static im_status run_levels(im_sketch* sk, int mode, bool all_first) {
         a.all_changed = 0;
         a.claim = claim + t;
         a.gen_next = ++sk->gen_counter;
-        a.fmt_in = sk->fmt.as<uint8_t>() + t;
-        a.fmt_out = sk->fmt.as<uint8_t>() + t + 1;
-        a.fmt_prev = sk->fmt.as<uint8_t>() + t - 1;
+        a.fmt_in = fmt + t;
+        a.fmt_out = fmt + t + 1;
+        a.fmt_prev = fmt + t - 1;
         CK(c, timed(c, mode == kPush ? kTPush : kTCover,
                     [&] { return launch_level(sk->kind, mode, sk->dev, a, grid, st); }));
     }
@@ -1137,7 +1165,7 @@ static im_status propagate(im_sketch* sk) {
     im_ctx* c = sk->ctx;
     CKS(phase_begin(sk, kPush));
     LevelArgs a = level_args(sk);
-    ulonglong2* ctr = sk->ctr.as<ulonglong2>();
+    ulonglong2* ctr = cur_ctr(sk);
     a.ql_out = sk->ql[0].as<QEntry>();
     a.cl_out = &ctr[0].x;
     a.qh_out = sk->qh[0].as<QEntry>();
@@ -1152,7 +1180,6 @@ static im_status propagate(im_sketch* sk) {
 static im_status incremental_rebuild(im_sketch* sk) {
     im_ctx* c = sk->ctx;
     auto st = c->stream;
-    ulonglong2* ctr = sk->ctr.as<ulonglong2>();
     IncrArgs x{};
     x.nv = sk->nv.as<uint32_t>();
     x.salt = sk->salt.as<uint32_t>();
@@ -1169,12 +1196,12 @@ static im_status incremental_rebuild(im_sketch* sk) {
     x.words_list = words_list_ok(sk) ? 1 : 0;
     x.awl = sk->awl.as<uint32_t>();
     x.awl_count = sk->awlc.as<unsigned int>();
-    if (x.words_list) CK(c, cudaMemsetAsync(sk->awlc.p, 0, 4, st));
     // 1. the affected registers (level 0 in bucket format where the sketch
     // has bucketed lists)
     CKS(phase_begin(sk, kAffect, x.buckets));
     LevelArgs a = level_args(sk);
     set_lcm(a, sk, kAffect);
+    ulonglong2* ctr = cur_ctr(sk);
     a.ql_out = sk->ql[0].as<QEntry>();
     a.cl_out = &ctr[0].x;
     a.qh_out = sk->qh[0].as<QEntry>();
@@ -1186,8 +1213,6 @@ static im_status incremental_rebuild(im_sketch* sk) {
     // affected chunks' out-buckets); 3. pull over their out-edges
     LevelArgs b = level_args(sk);
     set_lcm(b, sk, kCover);
-    CK(c, cudaMemsetAsync(x.list_count, 0, 4, st));
-    CK(c, cudaMemsetAsync(x.pctr, 0, 16, st));
     CK(c, timed(c, kTFill, [&] { return launch_incremental(1, sk->kind, sk->dev, b, x, st); }));
     if (sk->buckets && sk->pull_safe) {
         // the pull reads its queue's counters on the device
@@ -1214,6 +1239,7 @@ static im_status incremental_rebuild(im_sketch* sk) {
     CKS(phase_begin(sk, kPush, x.buckets));
     LevelArgs p = level_args(sk);
     set_lcm(p, sk, kPush);
+    ctr = cur_ctr(sk);
     p.ql_out = sk->ql[0].as<QEntry>();
     p.cl_out = &ctr[0].x;
     p.qh_out = sk->qh[0].as<QEntry>();
@@ -1221,9 +1247,9 @@ static im_status incremental_rebuild(im_sketch* sk) {
     p.chg_next = chg_buf(sk, kPush, 0).as<uint32_t>();
     CK(c, timed(c, kTOther, [&] { return launch_incremental(3, sk->kind, sk->dev, p, x, st); }));
     CKS(run_levels(sk, kPush, false));
-    // 5. the next rebuild starts from what covers visit after this one
-    CK(c, cudaMemsetAsync(sk->nv.p, 0, sk->nv.bytes, st));
-    CK(c, cudaMemsetAsync(sk->aff.p, 0, sk->aff.bytes, st));
+    // 5. no affected registers before the next rebuild (listed words were zeroed
+    // as the propagation's level 0 read them)
+    if (!x.words_list) CK(c, cudaMemsetAsync(sk->aff.p, 0, sk->aff.bytes, st));
     return IM_OK;
 }
 
@@ -1546,7 +1572,7 @@ static PickArgs pick_args(im_sketch* sk, int k) {
     a.k = k;
     a.rp_out = sk->g->rp_out.as<int32_t>();
     a.q_cover = sk->ql[0].as<QEntry>();
-    a.ctr_cover = &sk->ctr.as<ulonglong2>()[0].x;
+    a.ctr_cover = &cur_ctr(sk)[0].x;
     a.chg0 = chg_buf(sk, kCover, 0).as<uint32_t>();
     a.count = sk->count.as<unsigned long long>();
     a.mark = 1;
@@ -1617,7 +1643,7 @@ extern "C" im_status im_sketch_cover(im_sketch* sk, int32_t s, uint64_t* count_o
     if (s < 0 || s >= sk->g->n) return fail(c, IM_E_RANGE, "vertex %d out of range", s);
     CKS(phase_begin(sk, kCover));
     CK(c, launch_cover_seed(sk->M.as<uint8_t>(), sk->J, s, sk->g->rp_out.as<int32_t>(),
-                            sk->ql[0].as<QEntry>(), &sk->ctr.as<ulonglong2>()[0].x,
+                            sk->ql[0].as<QEntry>(), &cur_ctr(sk)[0].x,
                             chg_buf(sk, kCover, 0).as<uint32_t>(), sk->count.as<unsigned long long>(),
                             sk->buckets ? sk->bk_end[1].as<uint32_t>() : nullptr, sk->J / 16, c->stream));
     CKS(run_levels(sk, kCover, false));
@@ -2134,7 +2160,7 @@ extern "C" im_status im_batch_select_seeds(im_batch* b, const int32_t* J, const 
             pa.out_est = oest.as<double>();
             pa.rp_out = b->g->rp_out.as<int32_t>();
             pa.q_cover = sk->ql[0].as<QEntry>();
-            pa.ctr_cover = &sk->ctr.as<ulonglong2>()[0].x;
+            pa.ctr_cover = &cur_ctr(sk)[0].x;
             pa.chg0 = chg_buf(sk, kCover, 0).as<uint32_t>();
             pa.gcount = sk->gcount;
             pa.err = sk->err.as<uint32_t>();

@@ -35,14 +35,12 @@ constexpr int kFBlock = 256;
 using StatT = uint32_t;
 // resident blocks per SM the frontier kernels are compiled for (register cap);
 // the work is latency-bound, so more resident warps hide more of it
-#ifndef IM_PHASE_MIN_BLOCKS
-#define IM_PHASE_MIN_BLOCKS 4
+#ifndef IM_PHASE_BLOCK
+#define IM_PHASE_BLOCK 512
 #endif
-#ifndef IM_LEVEL_MIN_BLOCKS
-#define IM_LEVEL_MIN_BLOCKS 4
-#endif
-constexpr int kPhaseMinBlocks = IM_PHASE_MIN_BLOCKS;
-constexpr int kLevelMinBlocks = IM_LEVEL_MIN_BLOCKS;
+constexpr int kPBlock = IM_PHASE_BLOCK;  // threads of a phase kernel's block (two blocks an SM)
+constexpr int kPhaseMinBlocks = 1024 / kPBlock;
+constexpr int kLevelMinBlocks = 4;
 
 __device__ __forceinline__ unsigned long long wsum(unsigned long long x) {
 #pragma unroll
@@ -818,7 +816,9 @@ struct InlineCand {
     bool ok = false;
     uint32_t b = 0u, start = 0u, len = 0u, bits = 0u;
 };
-constexpr int kChainCap = 32;        // continuation stack entries per warp
+constexpr int kChainCap = 32;        // continuation stack entries per warp (in the warp's keep words,
+                                     // which only the edge scans use)
+static_assert(kChainCap * sizeof(int4) <= 32 * kKeepWords * sizeof(uint32_t), "stack fits the keep words");
 constexpr uint32_t kChainMaxLen = 32;  // bucket entries a continuation may take (one batch)
 
 // One position of a bucket walk: bucket bkt (vertex u, chunk c), list entry
@@ -953,12 +953,11 @@ __device__ __forceinline__ void bucket_slice(const GraphDev& g, const LevelArgs&
                                              StatT& st_chunks, StatT& st_cas,
                                              StatT& st_new, StatT& st_batches,
                                              StatT& st_dealt, bool out_b, int chain,
-                                             bool all_bits) {
+                                             bool all_bits, int4* stk) {
     const int lane = (int)lane_id();
     const int words = a.words;
     const uint32_t C = (uint32_t)a.chunks;
     const int64_t nb = a.nbuckets;
-    __shared__ int4 sChain[kFBlock / 32][kChainCap];
     int sp = 0, chain_used = 0;
     const uint16_t* chg16 = reinterpret_cast<const uint16_t*>(a.chg_cur);
     const int64_t fend = min(E, b1 << 5);
@@ -1047,8 +1046,8 @@ __device__ __forceinline__ void bucket_slice(const GraphDev& g, const LevelArgs&
         InlineCand ic;
         bucket_pos<KIND, MODE>(g, a, f < fend, bkt, e, chb, st_chunks, st_cas, st_new, st_dealt, out_b, ic);
         if (chain > 0) {
-            chain_push(sChain[threadIdx.x >> 5], sp, ic, 1);
-            chain_drain<KIND, MODE>(g, a, sChain[threadIdx.x >> 5], sp, chain, chain_used, st_chunks, st_cas,
+            chain_push(stk, sp, ic, 1);
+            chain_drain<KIND, MODE>(g, a, stk, sp, chain, chain_used, st_chunks, st_cas,
                                     st_new, st_batches, st_dealt, out_b);
         }
     }
@@ -1233,7 +1232,8 @@ __device__ __forceinline__ void level_work(const GraphDev& g, const LevelArgs& a
             const int64_t b0 = unit * lb;
             const int64_t b1 = min(nbl, b0 + lb);
             bucket_slice<KIND, MODE>(g, a, a.ql_in, b0, b1, nq, E, dense, ls.chunks, ls.cas, ls.fresh,
-                                     ls.batches, ls.bentries, out_b, chain, all_bits);
+                                     ls.batches, ls.bentries, out_b, chain, all_bits,
+                                     reinterpret_cast<int4*>(&sKeep[0][0]));
         }
         return;
     }
@@ -1383,7 +1383,7 @@ template <int KIND, int MODE>
 __global__ void __launch_bounds__(kFBlock, kLevelMinBlocks) k_level(GraphDev g, LevelArgs a) {
     __shared__ __align__(16) uint32_t sX[kMaxJ];
     __shared__ uint16_t sTab[kTabSize];
-    __shared__ uint32_t sKeep[kFBlock / 32][32][kKeepWords];
+    __shared__ __align__(16) uint32_t sKeep[kFBlock / 32][32][kKeepWords];
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const unsigned long long cl = __ldcg(a.cl_in);
@@ -1403,8 +1403,13 @@ __global__ void __launch_bounds__(kFBlock, kLevelMinBlocks) k_level(GraphDev g, 
     flush_stats<MODE>(a, ls);
 }
 
-// Grid-wide barrier of a cooperative launch: arrival counter + generation
-// word.  Every wait is bounded by `limit_ns` of global time (0: a block that
+// Grid-wide barrier of a cooperative launch: one arrival counter that only
+// grows (the blocks wait for gridDim * barriers passed), so the last arrival
+// itself releases the waiting blocks: no reset, no second word, no second
+// atomic.  Alone it takes 1.36 us over 304 blocks of 512 threads; arrival
+// counter, generation word and their fences over 608 blocks of 256 took 2.08
+// (304 blocks: 2.01; 152 blocks of 1024: 1.21, but large levels ran no
+// faster).  Every wait is bounded by `limit_ns` of global time (0: a block that
 // has to wait gives up at its first poll); a block that gives up raises
 // kErrBarrier and the abort word, and all blocks leave the phase at their
 // next barrier.
@@ -1414,42 +1419,39 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-__device__ bool grid_barrier(unsigned int* arrive, volatile unsigned int* gen, volatile unsigned int* abort_flag,
-                             uint32_t* err, unsigned long long limit_ns, unsigned int g0) {
-    // one arrival counter (the last block to arrive resets it and advances
-    // the generation); the waits poll only the generation word, with the
-    // abort word and the clock at the first poll and every 32nd
+__device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
+    unsigned int v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// target: arrivals that complete this barrier (gridDim * its number from 1).
+__device__ __forceinline__ bool grid_barrier(unsigned int* arrive, unsigned int target, volatile unsigned int* abort_flag,
+                                             uint32_t* err, unsigned long long limit_ns) {
     __syncthreads();
-    __shared__ bool ok;
+    __shared__ bool ok;  // (not __syncthreads_and: its uniform result costs the level loop 100 bytes of spills)
     if (threadIdx.x == 0) {
         ok = true;
-        // g0: the generation word's value before this barrier (it counts the
-        // barriers passed, so the caller knows it without a read)
-        __threadfence();
-        bool last = false;
-        if (atomicAdd(arrive, 1u) == gridDim.x - 1u) {
-            *arrive = 0u;
-            __threadfence();
-            atomicAdd((unsigned int*)gen, 1u);
-            last = true;
-        }
-        if (!last) {
-            const unsigned long long t0 = global_ns();
-            unsigned int it = 0;
-            while (*gen == g0) {
-                if ((it++ & 31u) == 0u) {
-                    if (*abort_flag) { ok = false; break; }
-                    if (global_ns() - t0 >= limit_ns) {
-                        atomicOr(err, kErrBarrier);
-                        *abort_flag = 1u;
-                        ok = false;
-                        break;
-                    }
+        // release: the block's writes (ordered before by the block barrier)
+        // are visible to whoever sees the arrival
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrive) : "memory");
+        unsigned int it = 0;
+        unsigned long long t0 = 0;
+        while ((int)(ld_acquire(arrive) - target) < 0) {
+            // the abort word and the clock at the first poll and every 32nd
+            if ((it & 31u) == 0u) {
+                const unsigned long long now = global_ns();
+                if (it == 0u) t0 = now;
+                if (*abort_flag) { ok = false; break; }
+                if (now - t0 >= limit_ns) {
+                    atomicOr(err, kErrBarrier);
+                    *abort_flag = 1u;
+                    ok = false;
+                    break;
                 }
-                __nanosleep(32);
             }
+            ++it;
         }
-        __threadfence();
     }
     __syncthreads();
     return ok;
@@ -1458,22 +1460,42 @@ __device__ bool grid_barrier(unsigned int* arrive, volatile unsigned int* gen, v
 // All levels of one phase in one cooperative launch: level t uses queue
 // buffers t % 3 as in k_level; a grid barrier separates levels; the phase
 // ends when both queues of the next level are empty.  BK as in level_work.
+// The level counters, work counters and barrier words of a launch must start
+// zeroed: launches alternate between two sets of them, and each launch zeroes
+// what the previous one used in the other set.  (18 memsets a pick and rebuild
+// were a fifth of a tiny selection: 10,000 vertices, J = 64, K = 10, 2.01 ms
+// with them, 1.66 ms without and with the shorter barrier.)
 template <int KIND, int MODE, bool BK>
-__global__ void __launch_bounds__(kFBlock, kPhaseMinBlocks) k_phase(GraphDev g, PhaseArgs p) {
+__global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, PhaseArgs p) {
     __shared__ __align__(16) uint32_t sX[kMaxJ];
     __shared__ uint16_t sTab[kTabSize];
-    __shared__ uint32_t sKeep[kFBlock / 32][32][kKeepWords];
+    __shared__ __align__(16) uint32_t sKeep[kPBlock / 32][32][kKeepWords];
+    // an earlier phase of this sketch gave up (the selection fails): its
+    // counters are not in order
+    if (__syncthreads_or(threadIdx.x == 0 && (*(volatile uint32_t*)p.base.err & (kErrBarrier | kErrLevels)) != 0u)) return;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     LevelArgs a = p.base;
     load_tables(a, sX, sTab);
+    if (p.bar_old && blockIdx.x == gridDim.x - 1) {
+        const int used = min((int)__ldcg(p.bar_old + kBarLevels) + 2, kMaxLevels + 2);
+        for (int i = threadIdx.x; i < used; i += blockDim.x) {
+            p.ctr_old[i] = make_ulonglong2(0ull, 0ull);
+            p.claim_old[i] = 0u;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < kBarWords; i += blockDim.x) p.bar_old[i] = 0u;
+    }
+    if (p.fmt && blockIdx.x == 0 && threadIdx.x == 0) p.fmt[0] = (uint8_t)p.fmt0;
+    unsigned int* const arrive = p.bar + kBarArrive;
+    unsigned int* const abort_flag = p.bar + kBarAbort;
     LevelStats ls;
     int t = 0;
     if (p.level_ns && blockIdx.x == 0 && threadIdx.x == 0) p.level_ns[0] = global_ns();
     // counters and format of the level's input queue, read once after the
     // barrier that precedes it
     unsigned long long pre_l = __ldcg(&p.ctr[0].x), pre_h = __ldcg(&p.ctr[0].y);
-    int pre_f = p.fmt != nullptr ? (int)__ldcg(p.fmt) : kFmtVertex;
+    int pre_f = p.fmt != nullptr ? p.fmt0 : kFmtVertex;
     // the previous level's input counters and format (its bits are cleared now)
     unsigned long long prev_l = 0ull, prev_h = 0ull;
     int prev_f = kFmtVertex;
@@ -1512,8 +1534,7 @@ __global__ void __launch_bounds__(kFBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
         prev_l = pre_l;
         prev_h = pre_h;
         prev_f = pre_f;
-        if (!grid_barrier(p.bar_arrive, p.bar_gen, p.abort_flag, a.err, p.limit_ns, (unsigned int)t))
-            break;
+        if (!grid_barrier(arrive, gridDim.x * (unsigned int)(t + 1), abort_flag, a.err, p.limit_ns)) break;
         if (p.level_ns && blockIdx.x == 0 && threadIdx.x == 0) p.level_ns[t + 1] = global_ns();
         pre_l = __ldcg(&p.ctr[t + 1].x);
         pre_h = __ldcg(&p.ctr[t + 1].y);
@@ -1522,7 +1543,7 @@ __global__ void __launch_bounds__(kFBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
     }
     // the last queue read (t - 1) still has its change bits; clearing them
     // leaves every change mask zero for the next phase
-    if (t >= 1 && t < p.max_levels && !*(volatile unsigned int*)p.abort_flag) {
+    if (t >= 1 && t < p.max_levels && !*(volatile unsigned int*)abort_flag) {
         const int bl = (t - 1) % 3;
         a.ql_prev = p.ql[bl];
         a.cl_prev = &p.ctr[t - 1].x;
@@ -1534,7 +1555,7 @@ __global__ void __launch_bounds__(kFBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
     }
     flush_stats<MODE>(a, ls);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *p.levels_out = t;
+        p.bar[kBarLevels] = (unsigned int)t;
         // a frontier that did not empty within the level limit is an error the
         // host reads with the others (it may read it only after later launches)
         if (t >= p.max_levels) atomicOr(a.err, kErrLevels);
@@ -1548,21 +1569,21 @@ int phase_grid() {
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_phase<kWC, kPush, true>, kFBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_phase<kWC, kPush, true>, kPBlock, 0);
         int pc = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pc, k_phase<kWC, kCover, true>, kFBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pc, k_phase<kWC, kCover, true>, kPBlock, 0);
         if (pc < per_sm) per_sm = pc;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pc, k_phase<kWC, kAffect, true>, kFBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pc, k_phase<kWC, kAffect, true>, kPBlock, 0);
         if (pc < per_sm) per_sm = pc;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pc, k_phase<kTrivalency, kPush, false>, kFBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pc, k_phase<kTrivalency, kPush, false>, kPBlock, 0);
         if (pc < per_sm) per_sm = pc;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pc, k_phase<kWC, kCover, false>, kFBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pc, k_phase<kWC, kCover, false>, kPBlock, 0);
         if (pc < per_sm) per_sm = pc;
         for (int kd : {0, 2, 3}) {
             int q = 0;
-            if (kd == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_phase<kUniform, kPush, true>, kFBlock, 0);
-            if (kd == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_phase<kTrivalency, kPush, true>, kFBlock, 0);
-            if (kd == 3) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_phase<kExplicit, kPush, true>, kFBlock, 0);
+            if (kd == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_phase<kUniform, kPush, true>, kPBlock, 0);
+            if (kd == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_phase<kTrivalency, kPush, true>, kPBlock, 0);
+            if (kd == 3) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, k_phase<kExplicit, kPush, true>, kPBlock, 0);
             if (q < per_sm) per_sm = q;
         }
         if (per_sm < 1 || !coop) per_sm = 0;
@@ -1577,7 +1598,7 @@ static cudaError_t coop_launch(const GraphDev& g, const PhaseArgs& p, int grid, 
     // edge-scan sketches (no bucketed lists) run the variant without the bucket code
     const void* fn = p.base.bk_end != nullptr ? (const void*)k_phase<KIND, MODE, true>
                                               : (const void*)k_phase<KIND, MODE, false>;
-    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kFBlock), args, 0, st);
+    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kPBlock), args, 0, st);
 }
 
 cudaError_t launch_phase(int kind, int mode, const GraphDev& g, const PhaseArgs& p, int grid,
@@ -2017,10 +2038,10 @@ cudaError_t launch_init_queues(int kind, const GraphDev& g, const LevelArgs& a, 
 // (q, ctr, overflow word) and, with chg, the bits to that change mask.  The
 // warp's (vertex, chunk) items are dealt one per lane (their bucket bounds
 // load in parallel); one reservation per warp keeps queue order and edge
-// offsets in step.
+// offsets in step.  consume: the vertices' bits are zeroed at the end.
 __device__ __forceinline__ void bucket_level0(const LevelArgs& a, bool valid, int32_t v,
-                                              const uint32_t* __restrict__ bits, uint32_t* chg, QEntry* q,
-                                              unsigned long long* ctr, unsigned long long* overflow) {
+                                              uint32_t* bits, uint32_t* chg, QEntry* q,
+                                              unsigned long long* ctr, unsigned long long* overflow, bool consume = false) {
     const int lane = (int)lane_id();
     uint32_t cm_lo = 0u, cm_hi = 0u;
     if (valid)
@@ -2112,6 +2133,11 @@ __device__ __forceinline__ void bucket_level0(const LevelArgs& a, bool valid, in
         slot += __popc(m);
         off += __shfl_sync(0xFFFFFFFFu, lincl, 31);
     }
+    if (consume) {
+        __syncwarp();  // every lane has read its items' bits
+        if (nch)
+            for (int w = 0; w < a.words; ++w) bits[(size_t)v * a.words + w] = 0u;
+    }
 }
 
 // Level-0 vertex entry of v whose change bits are `bits` (one thread): the
@@ -2135,21 +2161,31 @@ __device__ __forceinline__ void vertex_level0(const GraphDev& g, const LevelArgs
     want = true;
 }
 
-// Level 0 of the affected-set search: the newly visited registers (nv).
+// Level 0 of the affected-set search: the newly visited registers (nv), zeroed
+// as they are read (the next rebuild starts from what covers visit after this
+// one).  The counters that the later steps add to start at zero here as well.
 template <int KIND>
-__global__ void __launch_bounds__(kFBlock) k_affect_init(GraphDev g, LevelArgs a, const uint32_t* __restrict__ nv,
-                                                         int buckets) {
+__global__ void __launch_bounds__(kFBlock) k_affect_init(GraphDev g, LevelArgs a, IncrArgs x) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *x.list_count = 0u;
+        *x.awl_count = 0u;
+        x.pctr[0] = 0ull;
+        x.pctr[1] = 0ull;
+    }
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x; v0 < g.n; v0 += stride) {
         const int64_t v = v0 + threadIdx.x;
-        if (buckets) {
-            bucket_level0(a, v < g.n, (int32_t)v, nv, a.chg_next, a.ql_out, a.cl_out, a.ch_out);
+        if (x.buckets) {
+            bucket_level0(a, v < g.n, (int32_t)v, x.nv, a.chg_next, a.ql_out, a.cl_out, a.ch_out, true);
             continue;
         }
         bool want = false, heavy = false;
         int32_t rp = 0, deg = 0;
         uint32_t aux = 0u;
-        if (v < g.n) vertex_level0<KIND>(g, a, (int32_t)v, nv, want, rp, deg, aux, heavy, false);
+        if (v < g.n) {
+            vertex_level0<KIND>(g, a, (int32_t)v, x.nv, want, rp, deg, aux, heavy, false);
+            for (int w = 0; w < a.words; ++w) x.nv[(size_t)v * a.words + w] = 0u;
+        }
         append(want, (int32_t)v, rp, deg, aux, a.ql_out, a.cl_out, g.n, a.err);
     }
 }
@@ -2161,7 +2197,7 @@ __global__ void __launch_bounds__(kFBlock) k_affect_init(GraphDev g, LevelArgs a
 __global__ void __launch_bounds__(kFBlock) k_reset_affected(uint8_t* __restrict__ M, int32_t n, int J, int words,
                                                             const uint32_t* __restrict__ salt,
                                                             const int32_t* __restrict__ hkey,
-                                                            const uint32_t* __restrict__ aff, const int32_t* __restrict__ rp_out,
+                                                            uint32_t* aff, const int32_t* __restrict__ rp_out,
                                                             int32_t* __restrict__ list, int32_t* __restrict__ ldeg,
                                                             uint2* __restrict__ lmask, unsigned int* __restrict__ list_count,
                                                             LevelArgs o, QEntry* pq, unsigned long long* pctr) {
@@ -2369,13 +2405,14 @@ __global__ void __launch_bounds__(kFBlock) k_push_init_list(GraphDev g, LevelArg
 // + w (valid lanes) gives chunks 2w, 2w+1; each chunk whose 16 bits in `bits`
 // are nonzero and whose bucket (a's orientation) is nonempty is queued (its
 // bits in the entry's last word), and, with chg, its bits go to that change
-// mask.
+// mask.  consume: the words are zeroed once read.
 __device__ __forceinline__ void bucket_words(const LevelArgs& a, bool valid, uint32_t it,
-                                             const uint32_t* __restrict__ bits, uint32_t* chg, QEntry* q,
-                                             unsigned long long* ctr, unsigned long long* overflow) {
+                                             uint32_t* bits, uint32_t* chg, QEntry* q,
+                                             unsigned long long* ctr, unsigned long long* overflow, bool consume) {
     const int lane = (int)lane_id();
     const uint32_t v = valid ? it / (uint32_t)a.words : 0u, w = valid ? it % (uint32_t)a.words : 0u;
     const uint32_t word = valid ? __ldcg(bits + it) : 0u;
+    if (consume && valid) bits[it] = 0u;
     uint16_t* h16 = reinterpret_cast<uint16_t*>(chg);
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
@@ -2419,7 +2456,7 @@ __device__ __forceinline__ void bucket_words(const LevelArgs& a, bool valid, uin
 // Reset of the listed affected words to their vertices' own ranks (Alg. 1),
 // and the pull queue of their chunks' out-buckets (o: out orientation).
 __global__ void __launch_bounds__(kFBlock) k_reset_words(uint8_t* __restrict__ M, int J, const uint32_t* __restrict__ salt,
-                                                         const int32_t* __restrict__ hkey, const uint32_t* __restrict__ aff,
+                                                         const int32_t* __restrict__ hkey, uint32_t* aff,
                                                          const uint32_t* __restrict__ awl,
                                                          const unsigned int* __restrict__ awl_count, LevelArgs o,
                                                          QEntry* pq, unsigned long long* pctr) {
@@ -2439,12 +2476,13 @@ __global__ void __launch_bounds__(kFBlock) k_reset_words(uint8_t* __restrict__ M
                 M[(size_t)v * J + j] = (uint8_t)rank_of(ku, __ldg(salt + j));
             }
         }
-        bucket_words(o, valid, it, aff, nullptr, pq, pctr, pctr + 1);
+        bucket_words(o, valid, it, aff, nullptr, pq, pctr, pctr + 1, false);
     }
 }
 
 // Level 0 of the propagation after the pull from the listed words: their
-// chunks' in-buckets, the affected bits as the change mask.
+// chunks' in-buckets, the affected bits as the change mask.  The last reader of
+// the affected words: they are zeroed for the next rebuild.
 __global__ void __launch_bounds__(kFBlock) k_push_init_words(LevelArgs a, const uint32_t* __restrict__ awl,
                                                              const unsigned int* __restrict__ awl_count) {
     const int64_t cnt = (int64_t)__ldcg(awl_count);
@@ -2453,7 +2491,7 @@ __global__ void __launch_bounds__(kFBlock) k_push_init_words(LevelArgs a, const 
         const int64_t i = i0 + threadIdx.x;
         const bool valid = i < cnt;
         const uint32_t it = valid ? __ldcg(awl + i) : 0u;
-        bucket_words(a, valid, it, a.aff, a.chg_next, a.ql_out, a.cl_out, a.ch_out);
+        bucket_words(a, valid, it, a.aff, a.chg_next, a.ql_out, a.cl_out, a.ch_out, true);
     }
 }
 
@@ -2463,10 +2501,10 @@ cudaError_t launch_incremental(int step, int kind, const GraphDev& g, const Leve
     switch (step) {
         case 0:
             switch (kind) {
-                case kUniform: k_affect_init<kUniform><<<grid, kFBlock, 0, st>>>(g, a, x.nv, x.buckets); break;
-                case kWC: k_affect_init<kWC><<<grid, kFBlock, 0, st>>>(g, a, x.nv, x.buckets); break;
-                case kTrivalency: k_affect_init<kTrivalency><<<grid, kFBlock, 0, st>>>(g, a, x.nv, x.buckets); break;
-                default: k_affect_init<kExplicit><<<grid, kFBlock, 0, st>>>(g, a, x.nv, x.buckets); break;
+                case kUniform: k_affect_init<kUniform><<<grid, kFBlock, 0, st>>>(g, a, x); break;
+                case kWC: k_affect_init<kWC><<<grid, kFBlock, 0, st>>>(g, a, x); break;
+                case kTrivalency: k_affect_init<kTrivalency><<<grid, kFBlock, 0, st>>>(g, a, x); break;
+                default: k_affect_init<kExplicit><<<grid, kFBlock, 0, st>>>(g, a, x); break;
             }
             break;
         case 1:

@@ -133,14 +133,22 @@ struct PhaseArgs {
     int all_first;
     int max_levels;
     int32_t gen_base;                    // enqueue stamp of level t = gen_base + t
-    unsigned int* bar_arrive;            // groups arrived
-    unsigned int* bar_gen;
-    unsigned int* abort_flag;
+    unsigned int* bar;                   // barrier words (BarWord), zeroed before the launch
     unsigned long long limit_ns;         // bound on every barrier wait
-    int* levels_out;                     // levels the phase ran
     unsigned long long* level_ns;        // tracing: global time at the start of level t (may be NULL)
     uint8_t* fmt;                        // per level queue format (hybrid mode; NULL otherwise)
+    int fmt0;                            // format of the level-0 queue
+    // the counters and barrier words of the sketch's previous phase launch,
+    // which this launch zeroes (bar_old NULL: none)
+    ulonglong2* ctr_old;
+    unsigned int* claim_old;
+    unsigned int* bar_old;
 };
+
+// Barrier words of a phase launch (32-bit each): the arrival counter, polled
+// by the waiting blocks, on a 128-byte line of its own; the abort word; the
+// levels the phase ran.
+enum BarWord : int { kBarArrive = 0, kBarAbort = 32, kBarLevels = 33, kBarWords = 64 };
 
 int level_grid();
 int phase_grid();  // 0 when cooperative launch is unavailable
@@ -158,7 +166,7 @@ cudaError_t launch_init_queues(int kind, const GraphDev& g, const LevelArgs& a, 
 // 3 level-0 queue of the propagation from the list.  buckets: level-0 queues
 // of (vertex, chunk) buckets.
 struct IncrArgs {
-    const uint32_t* nv;
+    uint32_t* nv;
     const uint32_t* salt;
     const int32_t* hkey;
     int32_t* list;
@@ -176,7 +184,7 @@ struct IncrArgs {
     // the affected words listed by the search (bucket mode): steps 1 and 3
     // then walk only them (words_list)
     const uint32_t* awl;
-    const unsigned int* awl_count;
+    unsigned int* awl_count;
     int words_list;
 };
 cudaError_t launch_incremental(int step, int kind, const GraphDev& g, const LevelArgs& a, const IncrArgs& x,
