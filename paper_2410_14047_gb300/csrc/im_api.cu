@@ -1902,7 +1902,7 @@ extern "C" im_status im_spread_mc(im_graph* g, const int32_t* seeds, int32_t k, 
     if (e == cudaSuccess) e = cudaMemsetAsync(acc.p, 0, 16, st);
     if (e != cudaSuccess) { release(); return cuda_fail(c, e, "spread init"); }
     unsigned long long* cp = ctr.as<unsigned long long>();
-    const int grid = level_grid();
+    const int grid = mc_grid();
     int32_t stamp = 0;
     for (int64_t r0 = 0; r0 < R; r0 += B) {
         const int valid = (int)std::min<int64_t>(B, R - r0);

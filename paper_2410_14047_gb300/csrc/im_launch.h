@@ -360,6 +360,7 @@ struct McArgs {
     int32_t* gen;
     int32_t gen_next;
 };
+int mc_grid();
 cudaError_t launch_mc_level(int kind, const GraphDev& g, const McArgs& a, int grid,
                             cudaStream_t st);
 cudaError_t launch_mc_seed(const GraphDev& g, const McArgs& a, const int32_t* seeds, int k,
