@@ -48,19 +48,36 @@ __device__ __forceinline__ unsigned long long wsum(unsigned long long x) {
     return x;
 }
 
-// Last queue entry whose offset is <= f (warp-wide 32-ary search).
-__device__ __forceinline__ int32_t covering_entry(const QEntry* __restrict__ q, int32_t count, int64_t f) {
+// The queue window a warp starts a slice at: 32 consecutive entries (raw, one
+// a lane; a missing one starts past every position) that hold the entry
+// covering f0 and those of the 31 positions after it.  Returns the first
+// one's index.  A 32-ary search narrows the queue to 24 entries, and the
+// window is loaded there: only when the covering entry lies too far back in
+// it (a fifth of the slices at most) it is loaded again further on.  A
+// queue of 32 entries needs no search at all.  Each step is a dependent load,
+// of which a small level's time consists (R-MAT scale 17, J = 1024, K = 25: 6.62 ->
+// 6.57 ms; scale 20, weighted cascade: 103.6 -> 103.0 ms).
+__device__ __forceinline__ int32_t first_window(const QEntry* __restrict__ q, int32_t count, int64_t f0, int4& raw) {
     int32_t lo = 0, hi = count;
     const int lane = (int)lane_id();
-    while (hi - lo > 1) {
+    while (f0 > 0 && hi - lo > 24 && count > 32) {
         const int32_t step = (hi - lo + 31) >> 5;
         const int64_t idx = (int64_t)lo + (int64_t)step * (lane + 1);
-        const bool le = idx < hi && (int64_t)__ldcg(&q[idx].off) <= f;
+        const bool le = idx < hi && (int64_t)__ldcg(&q[idx].off) <= f0;
         const int c = __popc(__ballot_sync(0xFFFFFFFFu, le));
         const int32_t nlo = lo + step * c;
         const int32_t nhi = (c < 32) ? (int32_t)min((int64_t)hi, (int64_t)lo + (int64_t)step * (c + 1)) : hi;
         lo = nlo;
         hi = nhi;
+    }
+    raw = make_int4(0, 0, 0x7FFFFFFF, 0);
+    if (lo + lane < count) raw = __ldcg(reinterpret_cast<const int4*>(q) + lo + lane);
+    const bool past = lo + lane >= count || (int64_t)raw.z - f0 > 32;
+    if (!(__ballot_sync(0xFFFFFFFFu, past) >> 31)) {
+        // the window ends before position f0 + 33: start it at the covering entry
+        lo += __popc(__ballot_sync(0xFFFFFFFFu, (int64_t)raw.z - f0 <= 0)) - 1;
+        raw = make_int4(0, 0, 0x7FFFFFFF, 0);
+        if (lo + lane < count) raw = __ldcg(reinterpret_cast<const int4*>(q) + lo + lane);
     }
     return lo;
 }
@@ -418,8 +435,7 @@ __device__ __forceinline__ void dense_count_flush(const LevelArgs& a, StatT n) {
 // ---------------------------------------------------------------------------
 template <int KIND, int MODE>
 __device__ __forceinline__ void light_slice(const GraphDev& g, const LevelArgs& a, const QEntry* __restrict__ qlin,
-                                            const uint32_t* sX,
-                                            const uint16_t* sTab, int64_t b0, int64_t b1, int32_t nl,
+                                            const uint32_t* sX, int64_t b0, int64_t b1, int32_t nl,
                                             int64_t El, StatT& st_chunks,
                                             StatT& st_cas, StatT& st_new,
                                             StatT& st_batches, StatT& st_dealt,
@@ -429,10 +445,9 @@ __device__ __forceinline__ void light_slice(const GraphDev& g, const LevelArgs& 
     const int J = a.J, words = a.words;
     const int64_t fend = min(El, b1 << 5);
     int64_t f0 = b0 << 5;
-    int32_t qi = f0 == 0 ? 0 : covering_entry(qlin, nl, f0);
     // queue window of the first batch; later windows are prefetched one batch ahead
-    int4 raw = make_int4(0, 0, 0x7FFFFFFF, 0);
-    if (qi + lane < nl) raw = __ldcg(reinterpret_cast<const int4*>(qlin) + qi + lane);
+    int4 raw;
+    int32_t qi = first_window(qlin, nl, f0, raw);
     for (; f0 < fend; f0 += 32) {
         const int32_t wi = qi + lane;
         const bool wvalid = wi < nl;
@@ -966,8 +981,7 @@ __device__ __forceinline__ void bucket_slice(const GraphDev& g, const LevelArgs&
     int4 raw = make_int4(0, 0, 0x7FFFFFFF, 0);
     int64_t bk0 = 0;
     if (!dense) {
-        qi = f0 == 0 ? 0 : covering_entry(qlin, nq, f0);
-        if (qi + lane < nq) raw = __ldcg(reinterpret_cast<const int4*>(qlin) + qi + lane);
+        qi = first_window(qlin, nq, f0, raw);
     } else {
         bk0 = bucket_of_warp(a.bk_end, 0, nb, f0);
     }
@@ -1179,7 +1193,7 @@ struct UnitCursor {
 // registers).
 template <int KIND, int MODE, bool BK>
 __device__ __forceinline__ void level_work(const GraphDev& g, const LevelArgs& a, const uint32_t* sX,
-                                           const uint16_t* sTab, int64_t warp, LevelStats& ls,
+                                           int64_t warp, LevelStats& ls,
                                            uint32_t (*sKeep)[kKeepWords], unsigned long long cl,
                                            unsigned long long ch, int in_fmt, const ClearPlan& cp) {
     const bool in_b = in_fmt == kFmtBucket;
@@ -1330,14 +1344,14 @@ __device__ __forceinline__ void level_work(const GraphDev& g, const LevelArgs& a
             const int64_t lu = (int64_t)unit - nhv;
             const int64_t b0 = lu * lb;
             const int64_t b1 = min(nbl, b0 + lb);
-            light_slice<KIND, MODE>(g, a, ql, sX, sTab, b0, b1, nl, El, ls.chunks, ls.cas, ls.fresh,
+            light_slice<KIND, MODE>(g, a, ql, sX, b0, b1, nl, El, ls.chunks, ls.cas, ls.fresh,
                                     ls.batches, ls.dealt, ls.live, dense && nh > 0, sKeep, out_b, out_d,
                                     MODE == kPush && in_d ? &ls.chg : nullptr, draised, all_sims);
         } else {
             const int64_t hu = (int64_t)unit - nhv - lunits;
             const int64_t b0 = hu * lb;
             const int64_t b1 = min(nbh, b0 + lb);
-            light_slice<KIND, MODE>(g, a, a.qh_in, sX, sTab, b0, b1, nh, Eh, ls.chunks, ls.cas, ls.fresh,
+            light_slice<KIND, MODE>(g, a, a.qh_in, sX, b0, b1, nh, Eh, ls.chunks, ls.cas, ls.fresh,
                                     ls.batches, ls.dealt, ls.live, false, sKeep, out_b, false, nullptr, draised, false);
         }
     }
@@ -1372,9 +1386,10 @@ __device__ __forceinline__ void flush_stats(const LevelArgs& a, LevelStats& ls) 
     ls = LevelStats();
 }
 
-__device__ __forceinline__ void load_tables(const LevelArgs& a, uint32_t* sX, uint16_t* sTab) {
+// (The range table of the draws is not among them: a level tests the 16
+// simulations of a live chunk, whose masks were computed with the sketch.)
+__device__ __forceinline__ void load_tables(const LevelArgs& a, uint32_t* sX) {
     for (int i = threadIdx.x; i < a.J; i += blockDim.x) sX[i] = __ldg(a.X + i);
-    for (int i = threadIdx.x; i < kTabSize; i += blockDim.x) sTab[i] = __ldg(a.tab + i);
     __syncthreads();
 }
 
@@ -1382,7 +1397,6 @@ __device__ __forceinline__ void load_tables(const LevelArgs& a, uint32_t* sX, ui
 template <int KIND, int MODE>
 __global__ void __launch_bounds__(kFBlock, kLevelMinBlocks) k_level(GraphDev g, LevelArgs a) {
     __shared__ __align__(16) uint32_t sX[kMaxJ];
-    __shared__ uint16_t sTab[kTabSize];
     __shared__ __align__(16) uint32_t sKeep[kFBlock / 32][32][kKeepWords];
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1393,13 +1407,13 @@ __global__ void __launch_bounds__(kFBlock, kLevelMinBlocks) k_level(GraphDev g, 
         clear_prev_bits(a, warp, nwarps);
         return;
     }
-    load_tables(a, sX, sTab);
+    load_tables(a, sX);
     LevelStats ls;
     // the previous level's change bits (read by no one any more) are cleared
     // by the warps that find no work
     const ClearPlan cp = clear_plan(a, a.cl_prev ? __ldcg(a.cl_prev) : 0ull, a.ch_prev ? __ldcg(a.ch_prev) : 0ull,
                                     a.fmt_prev != nullptr ? (int)__ldcg(a.fmt_prev) : kFmtVertex);
-    level_work<KIND, MODE, true>(g, a, sX, sTab, warp, ls, sKeep[threadIdx.x >> 5], cl, ch, in_fmt, cp);
+    level_work<KIND, MODE, true>(g, a, sX, warp, ls, sKeep[threadIdx.x >> 5], cl, ch, in_fmt, cp);
     flush_stats<MODE>(a, ls);
 }
 
@@ -1468,7 +1482,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* arrive, unsigned int 
 template <int KIND, int MODE, bool BK>
 __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, PhaseArgs p) {
     __shared__ __align__(16) uint32_t sX[kMaxJ];
-    __shared__ uint16_t sTab[kTabSize];
     __shared__ __align__(16) uint32_t sKeep[kPBlock / 32][32][kKeepWords];
     // an earlier phase of this sketch gave up (the selection fails): its
     // counters are not in order
@@ -1476,7 +1489,7 @@ __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     LevelArgs a = p.base;
-    load_tables(a, sX, sTab);
+    load_tables(a, sX);
     if (p.bar_old && blockIdx.x == gridDim.x - 1) {
         const int used = min((int)__ldcg(p.bar_old + kBarLevels) + 2, kMaxLevels + 2);
         for (int i = threadIdx.x; i < used; i += blockDim.x) {
@@ -1530,7 +1543,7 @@ __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
         // the previous level's change bits are cleared by the warps that find
         // no work this level
         const ClearPlan cp = clear_plan(a, prev_l, prev_h, prev_f);
-        level_work<KIND, MODE, BK>(g, a, sX, sTab, warp, ls, sKeep[threadIdx.x >> 5], pre_l, pre_h, pre_f, cp);
+        level_work<KIND, MODE, BK>(g, a, sX, warp, ls, sKeep[threadIdx.x >> 5], pre_l, pre_h, pre_f, cp);
         prev_l = pre_l;
         prev_h = pre_h;
         prev_f = pre_f;
@@ -2008,8 +2021,15 @@ __global__ void __launch_bounds__(kFBlock) k_init_queues(GraphDev g, LevelArgs a
     }
 }
 
+// Blocks of a pass over `items` (one a thread), at most eight a multiprocessor:
+// a small graph's passes are launch time, and 1216 blocks of which a few find
+// work take about twice as long to launch and drain as those few alone.
+static int pass_grid(int64_t items) {
+    return (int)max((int64_t)1, min((int64_t)152 * 8, (items + kFBlock - 1) / kFBlock));
+}
+
 cudaError_t launch_init_queues(int kind, const GraphDev& g, const LevelArgs& a, cudaStream_t st) {
-    const int grid = 152 * 8;
+    const int grid = pass_grid(g.n);
     switch (kind) {
         case kUniform: k_init_queues<kUniform><<<grid, kFBlock, 0, st>>>(g, a); break;
         case kWC: k_init_queues<kWC><<<grid, kFBlock, 0, st>>>(g, a); break;
@@ -2497,7 +2517,8 @@ __global__ void __launch_bounds__(kFBlock) k_push_init_words(LevelArgs a, const 
 
 cudaError_t launch_incremental(int step, int kind, const GraphDev& g, const LevelArgs& a, const IncrArgs& x,
                                cudaStream_t st) {
-    const int grid = 152 * 8;
+    // the vertices (level 0), at most their words (lists)
+    const int grid = pass_grid(step == 0 ? (int64_t)g.n : (int64_t)g.n * a.words);
     switch (step) {
         case 0:
             switch (kind) {
@@ -2518,7 +2539,7 @@ cudaError_t launch_incremental(int step, int kind, const GraphDev& g, const Leve
             break;
         case 2: {
             if (!x.pull_buckets && x.count == 0) break;
-            const int pg = grid;
+            const int pg = 152 * 8;
             if (x.pull_buckets) {
                 k_pull_buckets<<<pg, kFBlock, 0, st>>>(a, x.pq, x.pctr);
                 break;
