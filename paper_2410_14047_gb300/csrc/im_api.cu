@@ -2132,6 +2132,7 @@ extern "C" im_status im_batch_select_seeds(im_batch* b, const int32_t* J, const 
         sk->gid = b->gid.as<int32_t>();
         sk->gcount = gcount_d.as<unsigned long long>();
         sk->gflag = flag_d.as<uint8_t>();
+        sk->defer = true;  // phases queue without host reads; the error word is read once, below
         if ((s = batch_build(sk)) != IM_OK) { cleanup(); return s; }
         ++builds;
         std::vector<unsigned long long> count((size_t)G, 0), oldcount((size_t)G, 0);
@@ -2190,6 +2191,7 @@ extern "C" im_status im_batch_select_seeds(im_batch* b, const int32_t* J, const 
                 ++builds;
             }
         }
+        if ((s = check_err(sk)) != IM_OK) { cleanup(); return s; }
         std::vector<int32_t> hseed((size_t)G * maxK);
         std::vector<double> hest((size_t)G * maxK);
         e = cudaMemcpyAsync(hseed.data(), oseed.p, hseed.size() * 4, cudaMemcpyDeviceToHost, st);
