@@ -1376,13 +1376,15 @@ static im_status build_buckets(im_sketch* sk) {
     if (s == IM_OK) s = dalloc(c, scan_tmp_bytes((int32_t)nb), tmp);
     if (s == IM_OK) s = dalloc(c, 16, ne);
     if (s != IM_OK) { drop(); return IM_OK; }  // no room: edge scans
+    const uint32_t* lcm_lo[2] = {sk->lcm_in_lo.as<uint32_t>(), sk->lcm_out_lo.as<uint32_t>()};
+    const uint32_t* lcm_hi[2] = {sk->lcm_in_hi.as<uint32_t>(), sk->lcm_out_hi.as<uint32_t>()};
     cudaError_t e = cudaMemsetAsync(ne.p, 0, 16, st);
     for (int o = 0; o < 2 && e == cudaSuccess; ++o) {
         e = cudaMemsetAsync(sk->bk_end[o].p, 0, sk->bk_end[o].bytes, st);
         if (e == cudaSuccess)
             e = timed(c, kTOther, [&] {
                 return launch_buckets(0, sk->kind, o == 0 ? kPush : kCover, sk->dev, sk->X.as<uint32_t>(),
-                                      sk->tab.as<uint16_t>(), J, sk->bk_end[o].as<uint32_t>(),
+                                      lcm_lo[o], lcm_hi[o], J, sk->bk_end[o].as<uint32_t>(),
                                       ne.as<unsigned long long>() + o, nullptr, nullptr, st);
             });
     }
@@ -1410,7 +1412,7 @@ static im_status build_buckets(im_sketch* sk) {
     for (int o = 0; o < 2 && e == cudaSuccess; ++o)
         e = timed(c, kTOther, [&] {
             return launch_buckets(1, sk->kind, o == 0 ? kPush : kCover, sk->dev, sk->X.as<uint32_t>(),
-                                  sk->tab.as<uint16_t>(), J, sk->bk_end[o].as<uint32_t>(), nullptr,
+                                  lcm_lo[o], lcm_hi[o], J, sk->bk_end[o].as<uint32_t>(), nullptr,
                                   sk->bk_other[o].as<int32_t>(), sk->bk_mask[o].as<uint16_t>(), st);
         });
     if (e != cudaSuccess) { drop(); return cuda_fail(c, e, "bucket fill"); }

@@ -241,7 +241,7 @@ __device__ __forceinline__ void red_add(unsigned long long* p, unsigned long lon
 
 // ---------------------------------------------------------------------------
 // Edge-balanced walks of a flat space split into rows (CSR edges, queue
-// entries): a warp takes kLcmEdgesPerWarp consecutive positions, finds the
+// entries): a warp takes up to kLcmEdgesPerWarp consecutive positions, finds the
 // row of the first by a 32-ary search of the row starts, then for each 32
 // positions loads the starts of the next 32 rows and every lane picks its row
 // among them (a lane whose position lies past those rows, after a run of
@@ -278,15 +278,18 @@ __device__ __forceinline__ int32_t row_of_thread(S&& start, int32_t lo, int32_t 
 
 // Edge-balanced walk of a flat space [0, m) split into rows by the
 // non-decreasing starts start(0..nrows) (start(0) = 0, start(nrows) = m), a
-// warp taking kLcmEdgesPerWarp consecutive positions; ALL: every lane calls
+// warp taking `per` consecutive positions; ALL: every lane calls
 // fn(f, row, valid) together, else fn(f, row) once per position.
 template <bool ALL, class S, class F>
 __device__ __forceinline__ void walk_rows_by(S&& start, int32_t nrows, int64_t m, F&& fn) {
     const int lane = (int)lane_id();
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t s0 = warp * kLcmEdgesPerWarp; s0 < m; s0 += nwarps * kLcmEdgesPerWarp) {
-        const int64_t s1 = min(m, s0 + kLcmEdgesPerWarp);
+    // a short space is spread over every warp of the grid, a batch of 32
+    // positions each at least
+    const int64_t per = min((int64_t)kLcmEdgesPerWarp, (((m + nwarps - 1) / nwarps + 31) >> 5) << 5);
+    for (int64_t s0 = warp * per; s0 < m; s0 += nwarps * per) {
+        const int64_t s1 = min(m, s0 + per);
         int32_t r0 = row_of_warp(start, 0, nrows, s0);
         for (int64_t f0 = s0; f0 < s1; f0 += 32) {
             const int64_t e = f0 + lane;
@@ -317,7 +320,7 @@ __device__ __forceinline__ void walk_rows_by(S&& start, int32_t nrows, int64_t m
 
 // Edge-balanced walk of a flat space [0, m) split into rows by the
 // non-decreasing starts rp[0..nrows] (rp[0] = 0, rp[nrows] = m): fn(f, row)
-// once per position, a warp taking kLcmEdgesPerWarp consecutive positions.
+// once per position.
 template <class F>
 __device__ __forceinline__ void walk_rows(const int32_t* __restrict__ rp, int32_t nrows, int64_t m, F&& fn) {
     walk_rows_by<false>([rp](int32_t r) -> int64_t { return (int64_t)__ldg(rp + r); }, nrows, m, fn);

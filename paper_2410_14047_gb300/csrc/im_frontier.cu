@@ -1688,27 +1688,6 @@ cudaError_t launch_level(int kind, int mode, const GraphDev& g, const LevelArgs&
 // ---------------------------------------------------------------------------
 // (kLcmEdgesPerWarp, row_of_warp and the row walks are in im_device.cuh.)
 
-// Live masks of one edge over every chunk that holds a candidate simulation:
-// fn(c, m16) for each chunk c with m16 != 0 (bit i: simulation 16c + i live).
-template <class F>
-__device__ __forceinline__ void edge_chunk_masks(uint32_t h, uint32_t thr, int J, const uint32_t* sX,
-                                                 const uint16_t* sTab, F&& fn) {
-    if (thr >= 0x80000000u) {
-        for (int c = 0; c < (J >> 4); ++c) fn(c, 0xFFFFu);
-        return;
-    }
-    if (thr == 0u) return;
-    int lo, hi;
-    candidate_range(h, thr, J, sX, sTab, lo, hi);
-    for (int c = lo >> 4; hi > lo && c <= ((hi - 1) >> 4); ++c) {
-        uint32_t m16 = 0u;
-        const int j1 = min(hi, 16 * c + 16);
-        for (int j = max(lo, 16 * c); j < j1; ++j)
-            if ((sX[j] ^ h) < thr) m16 |= 1u << (j - 16 * c);
-        if (m16) fn(c, m16);
-    }
-}
-
 // Chunks of one edge with at least one live simulation: bits c of lo (c <
 // 32) and hi (c >= 32).  A chunk's scan stops at its first live simulation
 // (sorted X puts an edge's candidates in a few consecutive chunks).
@@ -1788,58 +1767,168 @@ __global__ void __launch_bounds__(kFBlock) k_live_chunks(GraphDev g, const uint3
     });
 }
 
-// Bucketed live lists: pass 0 counts, pass 1 places (see launch_buckets).
-// Edges are walked in row order and a row's edges are sorted by hash, so the
-// lanes of a warp often share a bucket (same row, nearby simulations): the
-// count pass makes one atomic per bucket and chunk for those lanes together;
-// the place pass takes positions one entry at a time (its stores follow).
-template <int KIND, int MODE, int PASS>
-__global__ void __launch_bounds__(kFBlock) k_buckets(GraphDev g, const uint32_t* __restrict__ X,
-                                                     const uint16_t* __restrict__ tab, int J,
-                                                     uint32_t* __restrict__ cnt_or_end,
-                                                     int32_t* __restrict__ other_out,
-                                                     uint16_t* __restrict__ mask_out) {
-    __shared__ __align__(16) uint32_t sX[kMaxJ];
-    __shared__ uint16_t sTab[kTabSize];
-    load_sims(X, tab, J, sX, sTab);
-    const int C = J >> 4;
-    if constexpr (PASS == 1) {
-        for_each_edge<KIND, MODE>(g, [&](int64_t, int32_t v, int32_t other, uint32_t h, uint32_t thr) {
-            edge_chunk_masks(h, thr, J, sX, sTab, [&](int c, uint32_t m16) {
-                const uint32_t pos = atomicAdd(cnt_or_end + (int64_t)v * C + c, 1u);
-                other_out[pos] = other;
-                mask_out[pos] = (uint16_t)m16;
-            });
-        });
-        return;
+// 32 x 32 bit transpose over a warp: bit c of lane i becomes bit i of lane c.
+__device__ __forceinline__ uint32_t transpose32(uint32_t x) {
+    const unsigned lane = lane_id();
+    constexpr uint32_t keep[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const int j = 16 >> k;
+        const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, j);
+        x = (lane & j) ? ((x & ~keep[k]) | ((y & ~keep[k]) >> j)) : ((x & keep[k]) | ((y & keep[k]) << j));
     }
+    return x;
+}
+
+// The live simulations of chunk c for an edge of hash h and threshold thr, 16
+// bits: (x ^ h) < thr (both sides at most 2^31) is the sign of the
+// difference, shifted in one simulation after the other.
+__device__ __forceinline__ uint32_t live16(const uint32_t* sX, int c, uint32_t h, uint32_t thr) {
+    const uint4* xs = reinterpret_cast<const uint4*>(sX + c * 16);
+    uint32_t m = 0u;
+#pragma unroll
+    for (int w = 3; w >= 0; --w) {
+        const uint4 x = xs[w];
+        m = __funnelshift_l((x.w ^ h) - thr, m, 1);
+        m = __funnelshift_l((x.z ^ h) - thr, m, 1);
+        m = __funnelshift_l((x.y ^ h) - thr, m, 1);
+        m = __funnelshift_l((x.x ^ h) - thr, m, 1);
+    }
+    return m;
+}
+
+// Bucketed live lists (see launch_buckets), from the live chunk masks of the
+// orientation's edges: pass 0 counts every bucket's entries, pass 1 places them.
+//
+// Edges are walked in row order, 32 a step.  The step's chunk masks are
+// transposed, so that lane c holds the edges live in chunk c; a row's edges are
+// a run of lanes, and the row's entries in chunk c are the set bits of that
+// run: one reduction (pass 0) or one reservation (pass 1) per row and chunk
+// for all of them, 32 chunks at once on consecutive words.  The entries
+// themselves are then dealt one to each lane, their places known from the
+// reservation and the bits before them.  (Testing every candidate simulation in
+// both passes and reserving entry by entry, the two orientations of R-MAT scale
+// 19, trivalency, J = 512, took 1.01 ms to count and 0.93 ms to place; 0.27 and
+// 0.79 ms this way, the placing bound by its scattered 2- and 4-byte stores.)
+template <int MODE>
+__global__ void __launch_bounds__(kFBlock) k_bucket_count(GraphDev g, const uint32_t* __restrict__ lcm_lo,
+                                                          const uint32_t* __restrict__ lcm_hi, int C,
+                                                          uint32_t* __restrict__ cnt) {
+    const int32_t* rp = MODE == kPush ? g.rp_in : g.rp_out;
+    const int lane = (int)lane_id();
+    walk_rows_all([rp](int32_t r) -> int64_t { return (int64_t)__ldg(rp + r); }, g.n, g.m,
+                  [&](int64_t e, int32_t v, bool valid) {
+        const uint32_t lo = transpose32(valid ? __ldg(lcm_lo + e) : 0u);
+        const uint32_t hi = C > 32 ? transpose32(valid ? __ldg(lcm_hi + e) : 0u) : 0u;
+        const int32_t vp = __shfl_up_sync(0xFFFFFFFFu, v, 1);
+        unsigned heads = __ballot_sync(0xFFFFFFFFu, valid && (lane == 0 || v != vp));
+        while (heads) {
+            const int s = __ffs(heads) - 1;
+            heads &= heads - 1u;
+            const unsigned run = (heads ? (heads & (0u - heads)) - 1u : 0xFFFFFFFFu) & (0xFFFFFFFFu << s);
+            uint32_t* row = cnt + (int64_t)__shfl_sync(0xFFFFFFFFu, v, s) * C;
+            const int k0 = __popc(lo & run), k1 = __popc(hi & run);
+            if (lane < C && k0) atomicAdd(row + lane, (unsigned)k0);
+            if (lane + 32 < C && k1) atomicAdd(row + lane + 32, (unsigned)k1);
+        }
+    });
+}
+
+// Threads of a placing block: the reservations of a step (32 rows at most, C
+// chunks) stay in shared memory, 8 KB a warp for 64 chunks.
+static int place_block(int C) { return C > 32 ? 128 : kFBlock; }
+
+template <int KIND, int MODE>
+__global__ void __launch_bounds__(kFBlock) k_bucket_place(GraphDev g, const uint32_t* __restrict__ X,
+                                                          const uint32_t* __restrict__ lcm_lo,
+                                                          const uint32_t* __restrict__ lcm_hi, int J,
+                                                          uint32_t* __restrict__ cursor,
+                                                          int32_t* __restrict__ other_out,
+                                                          uint16_t* __restrict__ mask_out) {
+    __shared__ __align__(16) uint32_t sX[kMaxJ];
+    __shared__ uint32_t sBits[kFBlock / 32][64];  // transposed masks of the step
+    extern __shared__ uint32_t sBase[];           // [warp][row of the step][chunk]: the reserved place
+    for (int i = threadIdx.x; i < J; i += blockDim.x) sX[i] = __ldg(X + i);
+    __syncthreads();
+    const int C = J >> 4;
+    const int lane = (int)lane_id(), wib = threadIdx.x >> 5;
+    uint32_t* const base = sBase + (size_t)wib * 32 * C;
+    uint32_t* const bits = sBits[wib];
     const int32_t* rp = MODE == kPush ? g.rp_in : g.rp_out;
     walk_rows_all([rp](int32_t r) -> int64_t { return (int64_t)__ldg(rp + r); }, g.n, g.m,
                   [&](int64_t e, int32_t v, bool valid) {
-        uint32_t lo = 0u, hi = 0u;
+        uint32_t m_lo = 0u, m_hi = 0u, h = 0u, thr = 0u;
+        int32_t o = 0;
         if (valid) {
-            uint32_t h, thr;
+            m_lo = __ldg(lcm_lo + e);
+            if (C > 32) m_hi = __ldg(lcm_hi + e);
+            o = __ldg((MODE == kPush ? g.src_in : g.col_out) + e);
+            h = __ldg((MODE == kPush ? g.h_in : g.h_out) + e);
             if constexpr (MODE == kPush) {
-                const int32_t other = __ldg(g.src_in + e);
-                h = __ldg(g.h_in + e);
-                const uint32_t aux = KIND == kWC ? __ldg(g.thr_v + v) : 0u;
-                thr = edge_threshold<KIND, true>(g, (uint32_t)other, (uint32_t)v, e, aux);
+                if (KIND == kTrivalency && g.tri_b) {
+                    const int2 tb = __ldg(g.tri_b + v);
+                    const int cls = (e >= tb.x ? 1 : 0) + (e >= tb.y ? 1 : 0);
+                    thr = cls == 0 ? g.tri_thr[0] : (cls == 1 ? g.tri_thr[1] : g.tri_thr[2]);
+                } else {
+                    thr = edge_threshold<KIND, true>(g, (uint32_t)o, (uint32_t)v, e, KIND == kWC ? __ldg(g.thr_v + v) : 0u);
+                }
             } else {
-                const int32_t other = __ldg(g.col_out + e);
-                h = __ldg(g.h_out + e);
-                thr = edge_threshold<KIND, false>(g, (uint32_t)v, (uint32_t)other, e, 0u);
+                thr = edge_threshold<KIND, false>(g, (uint32_t)v, (uint32_t)o, e, 0u);
             }
-            edge_live_chunks(h, thr, J, sX, sTab, lo, hi);
         }
-        uint32_t ul = __reduce_or_sync(0xFFFFFFFFu, lo), uh = __reduce_or_sync(0xFFFFFFFFu, hi);
-        while (ul | uh) {
-            int c;
-            if (ul) { c = __ffs(ul) - 1; ul &= ul - 1; }
-            else { c = 32 + __ffs(uh) - 1; uh &= uh - 1; }
-            const bool mine = ((c < 32 ? lo >> c : hi >> (c - 32)) & 1u) != 0u;
-            const long long key = mine ? (long long)v * C + c : -1ll;
-            const unsigned grp = __match_any_sync(0xFFFFFFFFu, key);
-            if (mine && (int)lane_id() == __ffs(grp) - 1) atomicAdd(cnt_or_end + key, (unsigned)__popc(grp));
+        const uint32_t lo = transpose32(m_lo), hi = C > 32 ? transpose32(m_hi) : 0u;
+        __syncwarp();  // the previous step's places have been read
+        bits[lane] = lo;
+        bits[lane + 32] = hi;
+        const int32_t vp = __shfl_up_sync(0xFFFFFFFFu, v, 1);
+        const unsigned heads = __ballot_sync(0xFFFFFFFFu, valid && (lane == 0 || v != vp));
+        int r = 0;
+        for (unsigned hs = heads; hs; ++r) {
+            const int s = __ffs(hs) - 1;
+            hs &= hs - 1u;
+            const unsigned run = (hs ? (hs & (0u - hs)) - 1u : 0xFFFFFFFFu) & (0xFFFFFFFFu << s);
+            uint32_t* row = cursor + (int64_t)__shfl_sync(0xFFFFFFFFu, v, s) * C;
+            const int k0 = __popc(lo & run), k1 = __popc(hi & run);
+            if (lane < C && k0) base[r * C + lane] = atomicAdd(row + lane, (unsigned)k0);
+            if (lane + 32 < C && k1) base[r * C + lane + 32] = atomicAdd(row + lane + 32, (unsigned)k1);
+        }
+        __syncwarp();
+        // this lane's row of the step, and the row's edges before this one
+        const unsigned upto = heads & (0xFFFFFFFFu >> (31 - lane));
+        const int my_r = __popc(upto) - 1;
+        const unsigned before = valid ? ((1u << lane) - 1u) & (0xFFFFFFFFu << (31 - __clz(upto))) : 0u;
+        const int nch = __popc(m_lo) + __popc(m_hi);
+        int incl = nch;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, incl, s);
+            if (lane >= s) incl += y;
+        }
+        const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        const int excl = incl - nch;
+        for (int k0 = 0; k0 < total; k0 += 32) {
+            const int k = k0 + lane;
+            int i = 0;
+#pragma unroll
+            for (int s = 16; s >= 1; s >>= 1) {
+                const int ic = __shfl_sync(0xFFFFFFFFu, incl, i + s - 1);
+                if (ic <= k) i += s;
+            }
+            if (i > 31) i = 31;
+            const int ex_i = __shfl_sync(0xFFFFFFFFu, excl, i);
+            const uint32_t lo_i = __shfl_sync(0xFFFFFFFFu, m_lo, i);
+            const uint32_t hi_i = C > 32 ? __shfl_sync(0xFFFFFFFFu, m_hi, i) : 0u;
+            const int32_t o_i = __shfl_sync(0xFFFFFFFFu, o, i);
+            const uint32_t h_i = __shfl_sync(0xFFFFFFFFu, h, i);
+            const uint32_t t_i = __shfl_sync(0xFFFFFFFFu, thr, i);
+            const int r_i = __shfl_sync(0xFFFFFFFFu, my_r, i);
+            const unsigned b_i = __shfl_sync(0xFFFFFFFFu, before, i);
+            if (k < total) {
+                const int c = nth_chunk(lo_i, hi_i, k - ex_i);
+                const uint32_t pos = base[r_i * C + c] + (uint32_t)__popc(bits[c] & b_i);
+                other_out[pos] = o_i;
+                mask_out[pos] = (uint16_t)live16(sX, c, h_i, t_i);
+            }
         }
     });
 }
@@ -1904,7 +1993,7 @@ __global__ void __launch_bounds__(kFBlock) k_fill_rate(GraphDev g, uint64_t seed
 cudaError_t launch_fill_rate(int kind, const GraphDev& g, uint64_t seed, const uint32_t* X, const uint16_t* tab,
                              int J, unsigned long long* out, cudaStream_t st) {
     if (g.m == 0) return cudaSuccess;
-    const int64_t groups = (g.m + kLcmEdgesPerWarp - 1) / kLcmEdgesPerWarp;
+    const int64_t groups = (g.m + 31) / 32;
     const int64_t want = (groups + (kFBlock / 32) - 1) / (kFBlock / 32);
     const int grid = (int)max((int64_t)1, min(want, (int64_t)level_grid()));
     switch (kind) {
@@ -1928,22 +2017,33 @@ static cudaError_t live_chunks_mode(int kind, const GraphDev& g, const uint32_t*
     return cudaGetLastError();
 }
 
-template <int MODE, int PASS>
-static cudaError_t buckets_mode(int kind, const GraphDev& g, const uint32_t* X, const uint16_t* tab, int J,
-                                uint32_t* ce, int32_t* other, uint16_t* mask, int grid, cudaStream_t st) {
+template <int MODE>
+static cudaError_t place_mode(int kind, const GraphDev& g, const uint32_t* X, const uint32_t* lo, const uint32_t* hi,
+                              int J, uint32_t* cursor, int32_t* other, uint16_t* mask, cudaStream_t st) {
+    const int C = J >> 4, block = place_block(C);
+    const size_t shared = (size_t)(block / 32) * 32 * C * sizeof(uint32_t);
+    const int64_t want = ((g.m + 31) / 32 + block / 32 - 1) / (block / 32);
+    const int grid = (int)max((int64_t)1, min(want, (int64_t)152 * 8));
     switch (kind) {
-        case kUniform: k_buckets<kUniform, MODE, PASS><<<grid, kFBlock, 0, st>>>(g, X, tab, J, ce, other, mask); break;
-        case kWC: k_buckets<kWC, MODE, PASS><<<grid, kFBlock, 0, st>>>(g, X, tab, J, ce, other, mask); break;
-        case kTrivalency: k_buckets<kTrivalency, MODE, PASS><<<grid, kFBlock, 0, st>>>(g, X, tab, J, ce, other, mask); break;
-        default: k_buckets<kExplicit, MODE, PASS><<<grid, kFBlock, 0, st>>>(g, X, tab, J, ce, other, mask); break;
+        case kUniform: k_bucket_place<kUniform, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask); break;
+        case kWC: k_bucket_place<kWC, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask); break;
+        case kTrivalency: k_bucket_place<kTrivalency, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask); break;
+        default: k_bucket_place<kExplicit, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask); break;
     }
     return cudaGetLastError();
 }
 
 static int edge_walk_grid(const GraphDev& g) {
-    const int64_t groups = (g.m + kLcmEdgesPerWarp - 1) / kLcmEdgesPerWarp;
+    const int64_t groups = (g.m + 31) / 32;
     const int64_t want = (groups + (kFBlock / 32) - 1) / (kFBlock / 32);
     return (int)max((int64_t)1, min(want, (int64_t)level_grid()));
+}
+
+// Blocks of a pass over `items` (one a thread), at most eight a multiprocessor:
+// a small graph's passes are launch time, and 1216 blocks of which a few find
+// work take about twice as long to launch and drain as those few alone.
+static int pass_grid(int64_t items) {
+    return (int)max((int64_t)1, min((int64_t)152 * 8, (items + kFBlock - 1) / kFBlock));
 }
 
 // Nonzero entries of cnt[0..n) added to *out (one atomic per block).
@@ -1971,22 +2071,20 @@ __global__ void __launch_bounds__(kFBlock) k_count_nonzero(const uint32_t* __res
 }
 
 cudaError_t launch_buckets(int pass, int kind, int mode, const GraphDev& g, const uint32_t* X,
-                           const uint16_t* tab, int J, uint32_t* cnt_or_end, unsigned long long* nonempty,
-                           int32_t* other, uint16_t* mask, cudaStream_t st) {
+                           const uint32_t* lcm_lo, const uint32_t* lcm_hi, int J, uint32_t* cnt_or_end,
+                           unsigned long long* nonempty, int32_t* other, uint16_t* mask, cudaStream_t st) {
     if (g.m == 0) return cudaSuccess;
-    const int grid = edge_walk_grid(g);
-    cudaError_t e;
-    if (mode == kPush)
-        e = pass == 0 ? buckets_mode<kPush, 0>(kind, g, X, tab, J, cnt_or_end, other, mask, grid, st)
-                      : buckets_mode<kPush, 1>(kind, g, X, tab, J, cnt_or_end, other, mask, grid, st);
-    else
-        e = pass == 0 ? buckets_mode<kCover, 0>(kind, g, X, tab, J, cnt_or_end, other, mask, grid, st)
-                      : buckets_mode<kCover, 1>(kind, g, X, tab, J, cnt_or_end, other, mask, grid, st);
-    if (e != cudaSuccess || pass != 0) return e;
+    if (pass != 0)
+        return mode == kPush ? place_mode<kPush>(kind, g, X, lcm_lo, lcm_hi, J, cnt_or_end, other, mask, st)
+                             : place_mode<kCover>(kind, g, X, lcm_lo, lcm_hi, J, cnt_or_end, other, mask, st);
+    const int64_t want = ((g.m + 31) / 32 + kFBlock / 32 - 1) / (kFBlock / 32);
+    const int grid = (int)max((int64_t)1, min(want, (int64_t)152 * 8));
+    if (mode == kPush) k_bucket_count<kPush><<<grid, kFBlock, 0, st>>>(g, lcm_lo, lcm_hi, J >> 4, cnt_or_end);
+    else k_bucket_count<kCover><<<grid, kFBlock, 0, st>>>(g, lcm_lo, lcm_hi, J >> 4, cnt_or_end);
     // the nonempty buckets, counted after the pass (not by a contended
     // counter in it)
     const int64_t nb = (int64_t)g.n * (J >> 4);
-    k_count_nonzero<<<152 * 4, kFBlock, 0, st>>>(cnt_or_end, nb, nonempty);
+    k_count_nonzero<<<pass_grid((nb + 3) / 4), kFBlock, 0, st>>>(cnt_or_end, nb, nonempty);
     return cudaGetLastError();
 }
 
@@ -2019,13 +2117,6 @@ __global__ void __launch_bounds__(kFBlock) k_init_queues(GraphDev g, LevelArgs a
         append(want && !heavy, (int32_t)v, rp, deg, aux, a.ql_out, a.cl_out, g.n, a.err);
         append(want && heavy, (int32_t)v, rp, deg, aux, a.qh_out, a.ch_out, g.n, a.err);
     }
-}
-
-// Blocks of a pass over `items` (one a thread), at most eight a multiprocessor:
-// a small graph's passes are launch time, and 1216 blocks of which a few find
-// work take about twice as long to launch and drain as those few alone.
-static int pass_grid(int64_t items) {
-    return (int)max((int64_t)1, min((int64_t)152 * 8, (items + kFBlock - 1) / kFBlock));
 }
 
 cudaError_t launch_init_queues(int kind, const GraphDev& g, const LevelArgs& a, cudaStream_t st) {

@@ -1388,9 +1388,9 @@ __global__ void k_check_rows(const int32_t* __restrict__ rp, const int32_t* __re
     });
 }
 
-// Blocks of an edge-balanced walk over m positions (kLcmEdgesPerWarp a warp).
+// Blocks of an edge-balanced walk over m positions (at least 32 a warp).
 static int walk_grid(int64_t m) {
-    const int64_t warps = (m + kLcmEdgesPerWarp - 1) / kLcmEdgesPerWarp;
+    const int64_t warps = (m + 31) / 32;
     int64_t grid = (warps + kWarpsPerBlock - 1) / kWarpsPerBlock;
     if (grid > 152 * 16) grid = 152 * 16;
     return (int)(grid < 1 ? 1 : grid);

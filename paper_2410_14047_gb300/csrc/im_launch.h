@@ -283,13 +283,14 @@ cudaError_t launch_fill_rate(int kind, const GraphDev& g, uint64_t seed, const u
 cudaError_t launch_live_chunks(int kind, int mode, const GraphDev& g, const uint32_t* X, const uint16_t* tab,
                                int J, uint32_t* lo, uint32_t* hi, cudaStream_t st);
 // Bucketed live lists of one orientation (mode kPush: in-edges grouped by
-// target, kCover: out-edges grouped by source).  Pass 0 counts bucket sizes
+// target, kCover: out-edges grouped by source), from its edges' live chunk
+// masks (lcm_hi: chunks 32 and up, J > 512).  Pass 0 counts bucket sizes
 // into cnt[n * J/16] (zeroed by the caller) and non-empty buckets into
 // *nonempty; after an exclusive scan of cnt into end[] (end[nb] = total),
 // pass 1 fills other / mask and leaves end[b] = end of bucket b.
 cudaError_t launch_buckets(int pass, int kind, int mode, const GraphDev& g, const uint32_t* X,
-                           const uint16_t* tab, int J, uint32_t* cnt_or_end, unsigned long long* nonempty,
-                           int32_t* other, uint16_t* mask, cudaStream_t st);
+                           const uint32_t* lcm_lo, const uint32_t* lcm_hi, int J, uint32_t* cnt_or_end,
+                           unsigned long long* nonempty, int32_t* other, uint16_t* mask, cudaStream_t st);
 // Lazy pick: refreshes S_v of every unpicked v whose stored (lb[v], v) is
 // below (S_cand, cand) with S_cand fresh, then takes the least stored pair.
 cudaError_t launch_pick_lazy(const PickArgs& a, cudaStream_t st);
