@@ -49,6 +49,8 @@ enum QueueFormat : int { kFmtVertex = 0, kFmtBucket = 1, kFmtDense = 2 };
 
 // One frontier level (propagation sweep or cover level).  Queue t of a phase
 // lives in buffer t % 3; counters pack count << 38 | edges.
+constexpr uint32_t kNoBlockQueue = 0xFFFFFFFFu;
+
 struct LevelArgs {
     uint8_t* M;
     int J;
@@ -111,6 +113,9 @@ struct LevelArgs {
     uint8_t* fmt_out;
     const uint8_t* fmt_prev;
     int32_t bucket_div;                  // output in bucket format when input work * bucket_div < m
+    // shared-memory address of the block's output buffer (see block_append;
+    // kNoBlockQueue: entries go to the queue one warp at a time)
+    uint32_t sq = kNoBlockQueue;
     int32_t bq_guard;                    // check the bucket queue's fill before each append (huge graphs)
     int32_t vq_cap;                      // vertex queue capacity (n)
     uint32_t* aff;                       // incremental rebuild: affected (vertex, simulation) bits
