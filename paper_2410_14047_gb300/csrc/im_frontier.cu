@@ -1395,6 +1395,10 @@ __device__ __forceinline__ void level_work(const GraphDev& g, const LevelArgs& a
 
 template <int MODE>
 __device__ __forceinline__ void flush_stats(const LevelArgs& a, LevelStats& ls) {
+    // (a warp that found no work has nothing to sum)
+    if (!__any_sync(0xFFFFFFFFu, (ls.chunks | ls.cas | ls.fresh | ls.hsims | ls.batches | ls.dealt | ls.live |
+                                  ls.bentries | ls.chg) != 0u))
+        return;
     const unsigned long long chunks = wsum(ls.chunks), cas = wsum(ls.cas), fresh = wsum(ls.fresh),
                              hsims = wsum(ls.hsims), batches = wsum(ls.batches), dealt = wsum(ls.dealt),
                              live = wsum(ls.live), bentries = wsum(ls.bentries), chg = wsum(ls.chg);
@@ -1589,17 +1593,21 @@ __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
     __shared__ __align__(16) uint32_t sKeep[kPBlock / 32][32][kKeepWords];
     __shared__ __align__(16) unsigned int sQueue[4 + 4 * kBlockQueue];
     // an earlier phase of this sketch gave up (the selection fails): its
-    // counters are not in order
-    if (__syncthreads_or(threadIdx.x == 0 && (*(volatile uint32_t*)p.base.err & (kErrBarrier | kErrLevels)) != 0u)) return;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    LevelArgs a = p.base;
-    a.sq = (uint32_t)__cvta_generic_to_shared(sQueue);
+    // counters are not in order.  (The error word, the first counters and the
+    // simulations are fetched together: a phase of two small levels is little
+    // more than its dependent loads.)
+    const bool failed = threadIdx.x == 0 && (*(volatile uint32_t*)p.base.err & (kErrBarrier | kErrLevels)) != 0u;
+    unsigned long long pre_l = __ldcg(&p.ctr[0].x), pre_h = __ldcg(&p.ctr[0].y);
+    for (int i = threadIdx.x; i < p.base.J; i += blockDim.x) sX[i] = __ldg(p.base.X + i);
     if (threadIdx.x == 0) {
         sQueue[0] = 0u;
         sQueue[1] = kBlockQueue;
     }
-    load_tables(a, sX);
+    if (__syncthreads_or(failed)) return;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    LevelArgs a = p.base;
+    a.sq = (uint32_t)__cvta_generic_to_shared(sQueue);
     if (p.bar_old && blockIdx.x == gridDim.x - 1) {
         const int used = min((int)__ldcg(p.bar_old + kBarLevels) + 2, kMaxLevels + 2);
         for (int i = threadIdx.x; i < used; i += blockDim.x) {
@@ -1615,13 +1623,13 @@ __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
     LevelStats ls;
     int t = 0;
     if (p.level_ns && blockIdx.x == 0 && threadIdx.x == 0) p.level_ns[0] = global_ns();
-    // counters and format of the level's input queue, read once after the
-    // barrier that precedes it
-    unsigned long long pre_l = __ldcg(&p.ctr[0].x), pre_h = __ldcg(&p.ctr[0].y);
+    // counters (pre_l, pre_h) and format of the level's input queue, read once
+    // after the barrier that precedes it
     int pre_f = p.fmt != nullptr ? p.fmt0 : kFmtVertex;
     // the previous level's input counters and format (its bits are cleared now)
     unsigned long long prev_l = 0ull, prev_h = 0ull;
     int prev_f = kFmtVertex;
+    bool done = false;
     for (; t < p.max_levels; ++t) {
         const int bi = t % 3, bo = (t + 1) % 3, bp = (t + 2) % 3;
         a.ql_in = p.ql[bi];
@@ -1664,19 +1672,17 @@ __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
         pre_l = __ldcg(&p.ctr[t + 1].x);
         pre_h = __ldcg(&p.ctr[t + 1].y);
         pre_f = p.fmt != nullptr ? (int)__ldcg(p.fmt + t + 1) : kFmtVertex;
-        if ((pre_l >> kCountShift) == 0 && (pre_h >> kCountShift) == 0) { ++t; break; }
+        if ((pre_l >> kCountShift) == 0 && (pre_h >> kCountShift) == 0) { ++t; done = true; break; }
     }
     // the last queue read (t - 1) still has its change bits; clearing them
     // leaves every change mask zero for the next phase
-    if (t >= 1 && t < p.max_levels && !*(volatile unsigned int*)abort_flag) {
+    if (done) {
         const int bl = (t - 1) % 3;
         a.ql_prev = p.ql[bl];
-        a.cl_prev = &p.ctr[t - 1].x;
         a.qh_prev = p.qh[bl];
-        a.ch_prev = &p.ctr[t - 1].y;
         a.chg_prev = p.chg[bl];
-        a.fmt_prev = p.fmt ? p.fmt + t - 1 : nullptr;
-        clear_prev_bits(a, warp, nwarps);
+        const ClearPlan cp = clear_plan(a, prev_l, prev_h, prev_f);
+        for (int64_t u = warp; u < cp.units; u += nwarps) clear_unit(a, cp, u);
     }
     flush_stats<MODE>(a, ls);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
