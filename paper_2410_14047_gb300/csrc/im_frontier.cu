@@ -350,6 +350,33 @@ __device__ __forceinline__ void vertex_enqueue_finish(const GraphDev& g, const L
     if constexpr (MODE == kPush) append(want && heavy, o, q.rp, deg, q.aux, a.qh_out, a.ch_out, a.vq_cap, a.err);
 }
 
+// The words an affected-set search lists are collected by the block as well (the
+// same layout after the queue's entries: taken, first place that did not fit,
+// words); called by the lanes that have one.
+constexpr int kBlockWords = 2048;
+constexpr uint32_t kBlockWordsAt = 16u + 16u * kBlockQueue;
+
+__device__ __forceinline__ void list_word(const LevelArgs& a, uint32_t word) {
+    cooperative_groups::coalesced_group grp = cooperative_groups::coalesced_threads();
+    const unsigned k = grp.size(), r = grp.thread_rank();
+    unsigned int base = 0u;
+    if (a.sq != kNoBlockQueue) {
+        const uint32_t at = a.sq + kBlockWordsAt;
+        if (r == 0) {
+            asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(base) : "r"(at), "r"(k) : "memory");
+            if (base + k > kBlockWords) asm volatile("red.shared.min.u32 [%0], %1;" ::"r"(at + 4u), "r"(base) : "memory");
+        }
+        base = grp.shfl(base, 0);
+        if (base + k <= kBlockWords) {
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(at + 16u + 4u * (base + r)), "r"(word) : "memory");
+            return;
+        }
+    }
+    if (r == 0) base = atomicAdd(a.awl_count, k);
+    base = grp.shfl(base, 0);
+    a.awl[base + r] = word;
+}
+
 // Affected-set search (incremental rebuild): marks the simulations of
 // chunk c in which target o becomes affected (cand: 0xFF bytes where o is
 // reached along a live edge and its register is not visited); returns the
@@ -364,14 +391,8 @@ __device__ __forceinline__ uint32_t mark_affected(const LevelArgs& a, const uint
     const uint32_t old = atomicOr(a.aff + (size_t)o * a.words + (c >> 1), b16 << sh);
     const uint32_t fresh = b16 & ~(old >> sh) & 0xFFFFu;
     st_new += (unsigned)__popc(fresh);
-    if (old == 0u && a.awl) {
-        // the word's first bit: list it (one append for the lanes here together)
-        cooperative_groups::coalesced_group grp = cooperative_groups::coalesced_threads();
-        unsigned int base = 0u;
-        if (grp.thread_rank() == 0) base = atomicAdd(a.awl_count, grp.size());
-        base = grp.shfl(base, 0);
-        a.awl[base + grp.thread_rank()] = (uint32_t)o * (uint32_t)a.words + (c >> 1);
-    }
+    // the word's first bit: list it
+    if (old == 0u && a.awl) list_word(a, (uint32_t)o * (uint32_t)a.words + (c >> 1));
     return fresh;
 }
 
@@ -1432,6 +1453,23 @@ __device__ __forceinline__ void load_tables(const LevelArgs& a, uint32_t* sX) {
     __syncthreads();
 }
 
+// The block's output buffers: queue entries, then (WORDS) the words of a search.
+template <bool WORDS>
+struct QueueShared {
+    __align__(16) unsigned int queue[4 + 4 * kBlockQueue + (WORDS ? 4 + kBlockWords : 0)];
+
+    __device__ __forceinline__ void init() {
+        if (threadIdx.x == 0) {
+            queue[0] = 0u;
+            queue[1] = kBlockQueue;
+            if constexpr (WORDS) {
+                queue[4 + 4 * kBlockQueue] = 0u;
+                queue[5 + 4 * kBlockQueue] = kBlockWords;
+            }
+        }
+    }
+};
+
 // Moves the block's collected entries to the level's output queue (every
 // thread of the block; buckets: the queue holds bucket entries).
 __device__ __forceinline__ void block_flush(const LevelArgs& a, unsigned int* hdr, bool buckets) {
@@ -1498,6 +1536,22 @@ __device__ __forceinline__ void block_flush(const LevelArgs& a, unsigned int* hd
         if (buckets) atomicOr(a.ch_out, 1ull);
         else atomicOr(a.err, kErrQueue);
     }
+}
+
+// Appends the block's collected words to the search's list.
+__device__ __forceinline__ void words_flush(const LevelArgs& a, unsigned int* hdr) {
+    __shared__ unsigned int at;
+    __syncthreads();
+    const unsigned n = min(hdr[0], hdr[1]);
+    if (n == 0u) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        hdr[0] = 0u;
+        hdr[1] = kBlockWords;
+        at = atomicAdd(a.awl_count, n);
+    }
+    __syncthreads();
+    for (unsigned i = threadIdx.x; i < n; i += blockDim.x) a.awl[at + i] = hdr[4 + i];
 }
 
 // One level per launch (used when the host traces every level).
@@ -1591,7 +1645,7 @@ template <int KIND, int MODE, bool BK>
 __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, PhaseArgs p) {
     __shared__ __align__(16) uint32_t sX[kMaxJ];
     __shared__ __align__(16) uint32_t sKeep[kPBlock / 32][32][kKeepWords];
-    __shared__ __align__(16) unsigned int sQueue[4 + 4 * kBlockQueue];
+    __shared__ QueueShared<MODE == kAffect> sQueue;
     // an earlier phase of this sketch gave up (the selection fails): its
     // counters are not in order.  (The error word, the first counters and the
     // simulations are fetched together: a phase of two small levels is little
@@ -1599,15 +1653,12 @@ __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
     const bool failed = threadIdx.x == 0 && (*(volatile uint32_t*)p.base.err & (kErrBarrier | kErrLevels)) != 0u;
     unsigned long long pre_l = __ldcg(&p.ctr[0].x), pre_h = __ldcg(&p.ctr[0].y);
     for (int i = threadIdx.x; i < p.base.J; i += blockDim.x) sX[i] = __ldg(p.base.X + i);
-    if (threadIdx.x == 0) {
-        sQueue[0] = 0u;
-        sQueue[1] = kBlockQueue;
-    }
+    sQueue.init();
     if (__syncthreads_or(failed)) return;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     LevelArgs a = p.base;
-    a.sq = (uint32_t)__cvta_generic_to_shared(sQueue);
+    a.sq = (uint32_t)__cvta_generic_to_shared(sQueue.queue);
     if (p.bar_old && blockIdx.x == gridDim.x - 1) {
         const int used = min((int)__ldcg(p.bar_old + kBarLevels) + 2, kMaxLevels + 2);
         for (int i = threadIdx.x; i < used; i += blockDim.x) {
@@ -1663,7 +1714,10 @@ __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
         const ClearPlan cp = clear_plan(a, prev_l, prev_h, prev_f);
         bool out_b = false;
         level_work<KIND, MODE, BK>(g, a, sX, warp, ls, sKeep[threadIdx.x >> 5], pre_l, pre_h, pre_f, cp, out_b);
-        block_flush(a, sQueue, out_b);
+        block_flush(a, sQueue.queue, out_b);
+        if constexpr (MODE == kAffect) {
+            if (a.awl) words_flush(a, sQueue.queue + kBlockWordsAt / 4);
+        }
         prev_l = pre_l;
         prev_h = pre_h;
         prev_f = pre_f;
