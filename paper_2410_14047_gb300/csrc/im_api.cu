@@ -32,6 +32,8 @@ struct im_ctx {
     uint64_t peak = 0;
     bool custom_alloc = false;
     im_allocator alloc{};
+    imi::BlockShares* shares = nullptr;  // a server's worker: where its launches' blocks come from
+    int blocks = 0;                      // held of them by the query that runs
     cudaMemPool_t pool = nullptr;  // stream-ordered pool of a server worker (else the device default)
     std::unordered_map<void*, size_t> sizes;
     std::string err;
@@ -1049,6 +1051,12 @@ static im_status run_phase_persistent(im_sketch* sk, int mode, bool all_first, i
     return IM_OK;
 }
 
+// Blocks of a phase launch: every resident block (at most 2048), or a query's
+// share of them in a server.
+static int phase_blocks(const im_ctx* c, int grid) {
+    return std::min(grid, c->shares ? c->blocks : 64 * 32);
+}
+
 // Runs frontier levels until both queues are empty.  Level t reads queue
 // t % 3 with counters ctr[t], writes queue (t+1) % 3 with counters ctr[t+1],
 // and clears the change bits of queue (t+2) % 3 (read by level t-1).  The host
@@ -1058,8 +1066,7 @@ static im_status run_levels(im_sketch* sk, int mode, bool all_first) {
     im_ctx* c = sk->ctx;
     auto st = c->stream;
     if (c->tuning.persistent) {
-        // one cooperative grid of every resident block (at most 2048)
-        const int pgrid = std::min(phase_grid(), 64 * 32);
+        const int pgrid = phase_blocks(c, phase_grid());
         if (pgrid > 0) return run_phase_persistent(sk, mode, all_first, pgrid);
     }
     // per-level launches: the counters stay dirty, the level-0 format is in memory
@@ -1696,6 +1703,7 @@ static im_status select_seeds_impl(im_ctx* c, im_graph* g, int32_t K, int32_t J,
     };
     im_status s = ensure_out_cap(sk, K);
     if (s != IM_OK) return bail(s);
+    if (c->shares) c->blocks = c->shares->take();
     if ((s = build_registers(sk)) != IM_OK) return bail(s);
     const double t_build = now_ms();
     c->stats.ms_build = t_build - t0;
@@ -1710,6 +1718,7 @@ static im_status select_seeds_impl(im_ctx* c, im_graph* g, int32_t K, int32_t J,
         if (e == cudaSuccess) e = sync_collect(c);
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "read count"));
         const uint64_t count = c->pinned[0];
+        if (c->shares) c->blocks = c->shares->adjust(c->blocks);  // (nothing of this query is in flight)
         score[k] = (double)count / (double)J;
         const double tr = now_ms();
         ms_pc += tr - tk;
@@ -1798,11 +1807,14 @@ extern "C" im_status im_fill_rate(im_graph* g, int32_t J, uint64_t seed, const i
 // ---------------------------------------------------------------------------
 namespace imi {
 
-im_status ctx_create_worker(int device, cudaStream_t stream, cudaMemPool_t pool, im_ctx** out) {
+int resident_blocks() { return std::min(phase_grid(), 64 * 32); }
+
+im_status ctx_create_worker(int device, cudaStream_t stream, cudaMemPool_t pool, BlockShares* shares, im_ctx** out) {
     im_ctx* c = nullptr;
     CKS(im_ctx_create(device, stream, 0, nullptr, &c));
     c->pool = pool;
-    c->tuning.persistent = 0;
+    c->shares = shares;
+    c->tuning.persistent = shares ? 1 : 0;
     *out = c;
     return IM_OK;
 }
@@ -1813,8 +1825,16 @@ const char* ctx_error(const im_ctx* c) { return c->err.c_str(); }
 im_status select_seeds_on(im_ctx* c, im_graph* g, int32_t K, int32_t J, const im_model* model,
                           uint64_t seed, double rebuild_eps, int32_t* seeds_out, double* score_out,
                           double* estimate_out) {
-    return select_seeds_impl(c, g, K, J, model, seed, rebuild_eps, seeds_out, score_out,
-                             estimate_out, nullptr);
+    if (c->shares) c->shares->enter();
+    const im_status s = select_seeds_impl(c, g, K, J, model, seed, rebuild_eps, seeds_out, score_out, estimate_out,
+                                          nullptr);
+    if (c->shares) {
+        // a failed query may have phases in flight
+        if (s != IM_OK) cudaStreamSynchronize(c->stream);
+        c->shares->leave(c->blocks);
+        c->blocks = 0;
+    }
+    return s;
 }
 
 uint64_t query_bytes(const im_graph* g, int32_t J, int32_t K) {
