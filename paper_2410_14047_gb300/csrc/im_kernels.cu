@@ -1,3 +1,4 @@
+#include <algorithm>
 // Kernels of the sketch-based IM hot path for GB300 (sm_103a).
 //
 //   k_sims         per-simulation draws X_j, salt_j, FASST sort, range table   (Sec. 2.2, Sec. 4.1)
@@ -392,6 +393,24 @@ __device__ __forceinline__ Top2 group_top2(const PickArgs& a, int64_t g) {
 }
 
 
+// The block's two least pairs from its warps' (one warp, a lane each).
+__device__ __forceinline__ Top2 merge_warps(const unsigned long long* s1, const int32_t* u1,
+                                            const unsigned long long* s2, const int32_t* u2) {
+    Top2 t;
+    const int lane = (int)lane_id();
+    if (lane < kWarpsPerBlock) {
+        t.s1 = s1[lane]; t.u1 = u1[lane]; t.s2 = s2[lane]; t.u2 = u2[lane];
+    }
+#pragma unroll
+    for (int off = kWarpsPerBlock / 2; off >= 1; off >>= 1) {
+        const unsigned long long a1 = __shfl_xor_sync(0xFFFFFFFFu, t.s1, off), a2 = __shfl_xor_sync(0xFFFFFFFFu, t.s2, off);
+        const int32_t b1 = __shfl_xor_sync(0xFFFFFFFFu, t.u1, off), b2 = __shfl_xor_sync(0xFFFFFFFFu, t.u2, off);
+        t.insert(a1, b1);
+        t.insert(a2, b2);
+    }
+    return t;
+}
+
 // Block + grid reduction of the per-thread Top2 (last block by ticket), then
 // the seed record: out_seed / out_S / out_est[k], the seed bit, the next
 // lazy candidate, and (mark) the seed row visited + queued for the cover.
@@ -406,8 +425,8 @@ __device__ void pick_finish(const PickArgs& a, Top2 t) {
     t.warp_reduce();
     if (lane == 0) { sS1[wib] = t.s1; sU1[wib] = t.u1; sS2[wib] = t.s2; sU2[wib] = t.u2; }
     __syncthreads();
+    if (wib == 0) t = merge_warps(sS1, sU1, sS2, sU2);
     if (threadIdx.x == 0) {
-        for (int w = 1; w < kWarpsPerBlock; ++w) { t.insert(sS1[w], sU1[w]); t.insert(sS2[w], sU2[w]); }
         a.part_S[blockIdx.x] = t.s1;
         a.part_u[blockIdx.x] = t.u1;
         if (a.part_S2) { a.part_S2[blockIdx.x] = t.s2; a.part_u2[blockIdx.x] = t.u2; }
@@ -428,8 +447,8 @@ __device__ void pick_finish(const PickArgs& a, Top2 t) {
     __syncthreads();  // the shared arrays are reused
     if (lane == 0) { sS1[wib] = g.s1; sU1[wib] = g.u1; sS2[wib] = g.s2; sU2[wib] = g.u2; }
     __syncthreads();
+    if (wib == 0) g = merge_warps(sS1, sU1, sS2, sU2);
     if (threadIdx.x == 0) {
-        for (int w = 1; w < kWarpsPerBlock; ++w) { g.insert(sS1[w], sU1[w]); g.insert(sS2[w], sU2[w]); }
         fS = g.s1;
         fU = g.u1;
         *a.ticket = 0u;
@@ -569,6 +588,20 @@ __global__ void __launch_bounds__(kBlock) k_group_summaries(PickArgs a) {
     for (int64_t g = warp; g < a.ngroups; g += nwarps) group_top2(a, g);
 }
 
+// Record of group g (no pairs past the last group).
+struct GroupRecord {
+    unsigned long long s1 = ~0ull, s2 = ~0ull, pk = 0x7FFFFFFF7FFFFFFFull;
+};
+__device__ __forceinline__ GroupRecord group_record(const PickArgs& a, int64_t g) {
+    GroupRecord r;
+    if (g < a.ngroups) {
+        r.s1 = __ldcg(a.gsum + 4 * g);
+        r.s2 = __ldcg(a.gsum + 4 * g + 1);
+        r.pk = __ldcg(a.gsum + 4 * g + 2);
+    }
+    return r;
+}
+
 // Lazy pick (CELF-style, exact): S_u only grows during a selection (covers
 // turn registers into visited = 2^32, rebuilds lower the ranks of what stays
 // unvisited), so lb[v] <= S_v.  With S_c fresh for the candidate c, every
@@ -580,15 +613,17 @@ __global__ void __launch_bounds__(kBlock) k_group_summaries(PickArgs a) {
 // vertex's group is re-recorded by the last block (pick_finish).
 __global__ void __launch_bounds__(kBlock) k_pick_lazy(PickArgs a) {
     const int lane = (int)lane_id();
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int32_t c = __ldcg(a.cand);
+    // the first groups' records come with the candidate, not after its row
+    GroupRecord next = group_record(a, warp + (int64_t)lane * nwarps);
     unsigned long long Sc = 0;
     int32_t uc = -1;  // no candidate: nothing is refreshed
     if (c >= 0) {
         Sc = warp_row_sum(a.M, a.J, c);
         uc = c;
     }
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     unsigned refreshed = 0;  // rows refreshed by this warp
     Top2 t;
     // one group a lane; lane l of warp w takes group w + l * nwarps, so the
@@ -596,15 +631,9 @@ __global__ void __launch_bounds__(kBlock) k_pick_lazy(PickArgs a) {
     // together), go to different warps
     for (int64_t base = warp; base < a.ngroups; base += nwarps * 32) {
         const int64_t g = base + (int64_t)lane * nwarps;
-        unsigned long long s1 = ~0ull, s2 = ~0ull;
-        int32_t u1 = 0x7FFFFFFF, u2 = 0x7FFFFFFF;
-        if (g < a.ngroups) {
-            s1 = __ldcg(a.gsum + 4 * g);
-            s2 = __ldcg(a.gsum + 4 * g + 1);
-            const unsigned long long pk = __ldcg(a.gsum + 4 * g + 2);
-            u1 = (int32_t)(uint32_t)pk;
-            u2 = (int32_t)(uint32_t)(pk >> 32);
-        }
+        const unsigned long long s1 = next.s1, s2 = next.s2;
+        const int32_t u1 = (int32_t)(uint32_t)next.pk, u2 = (int32_t)(uint32_t)(next.pk >> 32);
+        next = group_record(a, g + nwarps * 32);
         const bool stale = g < a.ngroups && (s1 < Sc || (s1 == Sc && u1 < uc));
         if (!stale) {
             // no stale row: its two least pairs as recorded
@@ -655,15 +684,16 @@ cudaError_t launch_pick(const PickArgs& a, cudaStream_t st) {
 }
 
 int pick_lazy_grid(int32_t n) {
-    // one group a lane, and at least 2048 warps: the stale groups of a pick
-    // (spread over the warps by the group-to-lane mapping) are refreshed by as
-    // many warps as there are
+    // one group a lane, and up to 2048 warps while there are groups for them:
+    // the stale groups of a pick (spread over the warps by the group-to-lane
+    // mapping) are refreshed by as many warps as there are.  Fewer groups take
+    // fewer blocks: each of them costs a ticket and two partial pairs that the
+    // last one reads (Chung-Lu 54k, 425 groups, K = 27: 3.62 -> 3.56 ms).
     const int64_t groups = ((int64_t)n + kGroupRows - 1) / kGroupRows;
-    int64_t warps = (groups + 31) / 32;
-    if (warps < 2048) warps = 2048;
+    const int64_t warps = std::max((groups + 31) / 32, std::min<int64_t>(groups, 2048));
     int64_t grid = (warps + kWarpsPerBlock - 1) / kWarpsPerBlock;
     if (grid > 152 * 8) grid = 152 * 8;
-    return (int)grid;
+    return (int)(grid < 1 ? 1 : grid);
 }
 
 int pick_groups(int32_t n) { return (int)(((int64_t)n + kGroupRows - 1) / kGroupRows); }
