@@ -1280,76 +1280,94 @@ __global__ void __launch_bounds__(kBlock) k_sort_hist(const unsigned long long* 
     hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = (int32_t)h[threadIdx.x];
 }
 
-// Scatter of one pass: the tile's keys are first ranked stably by digit
-// (rounds of 256 keys in index order; inside a round, warps in order, lanes of
-// a digit by __match_any_sync) and placed in shared memory in digit order,
-// then written out from there: consecutive threads write a digit's keys to
-// consecutive global positions (runs of about kSortTile / 256 keys instead of
-// one key per store).
-__global__ void __launch_bounds__(kBlock) k_sort_scatter(
+// Scatter of one pass: the tile's keys are ranked stably by digit and placed in
+// shared memory in digit order, then written out from there: consecutive
+// threads write a digit's keys to consecutive global positions (runs of about
+// kSortTile / 256 keys instead of one key per store).  Each warp ranks its own
+// run of consecutive keys (32 a step, lanes of a digit by __match_any_sync,
+// its digit counts in shared memory), so the block meets only for the scans
+// over warps and digits; every key is loaded before the first is ranked.
+// (256 keys a round for the whole block, with four block barriers a round:
+// 422 us a pass over 32 million keys, 295 us this way; the load of that graph
+// 7.09 -> 5.74 ms.  64 registers: four blocks a multiprocessor.)
+__global__ void __launch_bounds__(kBlock, 4) k_sort_scatter(
     const unsigned long long* __restrict__ keys, const int32_t* __restrict__ vals, int64_t n, int shift,
-    int nblocks, const int32_t* __restrict__ hist, const int32_t* __restrict__ offs,
+    int nblocks, const int32_t* __restrict__ offs,
     unsigned long long* __restrict__ keys_out, int32_t* __restrict__ vals_out) {
     __shared__ unsigned long long sk[kSortTile];
     __shared__ int32_t sv[kSortTile];
-    __shared__ unsigned int wcount[kWarpsPerBlock][256];
-    __shared__ unsigned int run[256];    // keys of the digit placed so far (tile order)
-    __shared__ unsigned int start[256];  // first tile position of the digit
-    __shared__ unsigned int gbase[256];  // global position of the tile's first key of the digit
+    __shared__ unsigned int wcount[kWarpsPerBlock][256];  // a warp's keys of a digit, then those of the warps before
+    __shared__ unsigned int start[256];                   // first tile position of the digit
+    __shared__ unsigned int gbase[256];                   // global position of the digit's first key, less start
+    __shared__ unsigned int wtot[kWarpsPerBlock];
+    static_assert(kBlock == 256, "a thread a digit");
     const int lane = (int)lane_id(), w = threadIdx.x >> 5;
     const int d0 = threadIdx.x;
-    const unsigned cnt_d = (unsigned)hist[(int64_t)d0 * nblocks + blockIdx.x];
-    gbase[d0] = (unsigned)offs[(int64_t)d0 * nblocks + blockIdx.x];
-    run[d0] = 0u;
-    // exclusive scan of the tile's digit counts (one digit a thread)
-    start[d0] = cnt_d;
-    __syncthreads();
-    for (int o = 1; o < 256; o <<= 1) {
-        const unsigned x = d0 >= o ? start[d0 - o] : 0u;
-        __syncthreads();
-        start[d0] += x;
-        __syncthreads();
-    }
-    start[d0] -= cnt_d;
+    const unsigned goff = (unsigned)__ldg(offs + (int64_t)d0 * nblocks + blockIdx.x);
     const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    for (int r = 0; r < kSortItems; ++r) {
-        for (int d = lane; d < 256; d += 32) wcount[w][d] = 0u;
-        __syncthreads();
-        const int64_t i = base + (int64_t)r * kBlock + threadIdx.x;
-        const bool ok = i < n;
-        unsigned long long k = 0;
-        int32_t v = 0;
-        unsigned d = 256u + (unsigned)lane;  // distinct dummy digits for missing keys
-        if (ok) {
-            k = keys[i];
-            v = vals[i];
-            d = (unsigned)(k >> shift) & 0xFFu;
-        }
-        const unsigned peers = __match_any_sync(0xFFFFFFFFu, d);
-        const unsigned rank_w = __popc(peers & ((1u << lane) - 1u));
-        if (ok && rank_w == 0) wcount[w][d] = __popc(peers);
-        __syncthreads();
-        if (ok) {
-            unsigned before = 0;
-            for (int ww = 0; ww < w; ++ww) before += wcount[ww][d];
-            const unsigned pos = start[d] + run[d] + before + rank_w;
-            sk[pos] = k;
-            sv[pos] = v;
-        }
-        __syncthreads();
-        {
-            unsigned tot = 0;
-            for (int ww = 0; ww < kWarpsPerBlock; ++ww) tot += wcount[ww][threadIdx.x];
-            run[threadIdx.x] += tot;
-        }
-        __syncthreads();
+    const int64_t mine = base + (int64_t)w * (32 * kSortItems) + lane;
+    unsigned long long k[kSortItems];
+    int32_t v[kSortItems];
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const bool ok = mine + 32 * i < n;
+        k[i] = ok ? __ldcs(keys + mine + 32 * i) : 0ull;
+        v[i] = ok ? __ldcs(vals + mine + 32 * i) : 0;
     }
+    for (int d = lane; d < 256; d += 32) wcount[w][d] = 0u;
+    __syncwarp();
+    unsigned rank[kSortItems];  // place among the warp's keys of the digit
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const bool ok = mine + 32 * i < n;
+        const unsigned d = ok ? (unsigned)(k[i] >> shift) & 0xFFu : 256u + (unsigned)lane;  // a digit of its own
+        const unsigned peers = __match_any_sync(0xFFFFFFFFu, d);
+        const unsigned before = ok ? wcount[w][d] : 0u;
+        rank[i] = before + (unsigned)__popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+        if (ok && (peers & ((1u << lane) - 1u)) == 0u) wcount[w][d] = before + (unsigned)__popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    // the digit's keys in the warps before each warp, and before the digit
+    unsigned cnt = 0;
+#pragma unroll
+    for (int ww = 0; ww < kWarpsPerBlock; ++ww) {
+        const unsigned c = wcount[ww][d0];
+        wcount[ww][d0] = cnt;
+        cnt += c;
+    }
+    unsigned incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned x = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) wtot[w] = incl;
+    __syncthreads();
+    unsigned first = incl - cnt;
+#pragma unroll
+    for (int ww = 0; ww < kWarpsPerBlock; ++ww) first += ww < w ? wtot[ww] : 0u;
+    start[d0] = first;
+    gbase[d0] = goff - first;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        if (mine + 32 * i >= n) continue;
+        const unsigned d = (unsigned)(k[i] >> shift) & 0xFFu;
+        const unsigned pos = start[d] + wcount[w][d] + rank[i];
+        sk[pos] = k[i];
+        sv[pos] = v[i];
+    }
+    __syncthreads();
     const int tile_n = (int)min((int64_t)kSortTile, n - base);
-    for (int j = threadIdx.x; j < tile_n; j += kBlock) {
-        const unsigned long long k = sk[j];
-        const unsigned d = (unsigned)(k >> shift) & 0xFFu;
-        const unsigned pos = gbase[d] + (unsigned)j - start[d];
-        keys_out[pos] = k;
+#pragma unroll
+    for (int i = 0; i < kSortItems; ++i) {
+        const int j = i * kBlock + (int)threadIdx.x;
+        if (j >= tile_n) break;
+        const unsigned long long key = sk[j];
+        const unsigned pos = gbase[(unsigned)(key >> shift) & 0xFFu] + (unsigned)j;
+        keys_out[pos] = key;
         vals_out[pos] = sv[j];
     }
 }
@@ -1580,7 +1598,7 @@ cudaError_t launch_radix_sort(unsigned long long* keys, int32_t* vals, int64_t n
         k_sort_hist<<<nb, kBlock, 0, st>>>(ka, n, shift, nb, hist);
         cudaError_t e = launch_exclusive_scan(hist, cnt, offs, scan_tmp, st);
         if (e != cudaSuccess) return e;
-        k_sort_scatter<<<nb, kBlock, 0, st>>>(ka, va, n, shift, nb, hist, offs, kb, vb);
+        k_sort_scatter<<<nb, kBlock, 0, st>>>(ka, va, n, shift, nb, offs, kb, vb);
         unsigned long long* tk = ka; ka = kb; kb = tk;
         int32_t* tv = va; va = vb; vb = tv;
     }
