@@ -12,6 +12,8 @@
 // hub's edges are spread over many warps.
 #include <cstdio>
 
+#include <cuda_fp16.h>
+
 #include "im_launch.h"
 
 namespace im {
@@ -207,17 +209,103 @@ __device__ __forceinline__ unsigned long long row_terms16(uint4 q) {
     return ((unsigned long long)big << 32) + lo;
 }
 
-// Sum of the row owned by this lane's segment; valid in every lane of the segment.
-__device__ __forceinline__ unsigned long long row_sum(const uint8_t* __restrict__ M, int J,
-                                                      int32_t row, int lpr, int cpl, int seg_lane) {
-    unsigned long long s = 0;
-    const uint8_t* p = M + (size_t)row * J;
-    for (int c = 0; c < cpl; ++c) {
-        const int chunk = seg_lane + c * lpr;
-        s += row_terms16(__ldcg(reinterpret_cast<const uint4*>(p) + chunk));
+// The same terms on the tensor and FMA pipes.  Summed register by register the
+// estimate is bound by the integer ALU (about 100 operations a 16-byte piece,
+// ncu: ALU pipe 78 % busy at 2.7 TB/s); this way the pipes share the work (ALU
+// 42 %, FMA 38 %, tensor 16 %), and the issue slots and the warps in flight set
+// the pace: a million rows of 256 take 82.3 us, 91.3 before; 86.9 at three
+// blocks a multiprocessor (74 registers), 86.2 and 89.8 at five and six with one
+// row step in flight.
+//
+// A rank r (a visited register counts as rank 0: both are 2^32) becomes the
+// fp16 number 2^(15-r), whose bits are one subtraction for two registers: ranks
+// up to 29, a zero for 30; a piece with a larger one is summed register by
+// register.  Each number goes to one of two parts, 2^2 and above (ranks to 13)
+// or below: adding and subtracting 6144, whose last fp16 place is 4, leaves the
+// upper part.  A matrix product with ones then sums both parts over the pieces
+// of four lanes, in fp32 without rounding: at most 256 terms, multiples of 2^2
+// up to 2^15 (22 bits) or of 2^-14 up to 2 (24 bits).
+__device__ __forceinline__ uint32_t prmt(uint32_t x, uint32_t sel) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(x), "r"(sel));
+    return r;
+}
+
+// d[0], d[2]: the upper and lower sums of the quad's pieces; rare: bit 7 of a
+// byte set for a rank of 30 or more.
+__device__ __forceinline__ void add_terms16(uint4 q, float (&d)[4], uint32_t& rare) {
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    const __half2 big = __float2half2_rn(6144.f);
+    constexpr uint32_t ones = 0x3C003C00u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t r = w[i] & ~prmt(w[i], 0xBA98u);  // visited bytes to rank 0
+        rare |= r + 0x62626262u;
+        uint32_t hi[2], lo[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t bits = 0x78007800u - (prmt(r, h ? 0x4342u : 0x4140u) << 10);
+            const __half2 v = *reinterpret_cast<const __half2*>(&bits);
+            const __half2 up = __hsub2_rn(__hadd2_rn(v, big), big);
+            const __half2 dn = __hsub2_rn(v, up);
+            hi[h] = *reinterpret_cast<const uint32_t*>(&up);
+            lo[h] = *reinterpret_cast<const uint32_t*>(&dn);
+        }
+        // rows 0..7 of the matrix: the upper parts of the eight quads; rows 8..15: the lower
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %8}, "
+            "{%0, %1, %2, %3};"
+            : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+            : "r"(hi[0]), "r"(lo[0]), "r"(hi[1]), "r"(lo[1]), "r"(ones));
     }
+}
+
+// The rows of a warp step: rpw rows of lpr lanes, up to four pieces a lane, lpr
+// pieces apart (the lanes of a row read neighbouring pieces).
+__device__ __forceinline__ void load_row_pieces(const uint8_t* __restrict__ M, int J, int64_t row, int64_t limit,
+                                                int cpl, int lpr, int seg_lane, uint4 (&q)[4]) {
+    const uint4* p = reinterpret_cast<const uint4*>(M + (size_t)(row < limit ? row : 0) * J) + seg_lane;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        q[c] = (c < cpl && row < limit) ? __ldcs(p + c * lpr) : make_uint4(0u, 0u, 0u, 0u);
+}
+
+// S of the row owned by this lane's segment (whole warp; valid in every lane of
+// the segment).  From J = 64 on a row takes whole quads of lanes.
+__device__ __forceinline__ unsigned long long row_sum(const uint4 (&q)[4], int J, int cpl, int lpr) {
+    unsigned long long s = 0;
+    if (J >= 64) {
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        uint32_t rare = 0u;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (c < cpl) add_terms16(q[c], d, rare);
+        if (!__any_sync(0xFFFFFFFFu, (rare & 0x80808080u) != 0u)) {
+            // in units of 2^17: the upper sum is whole, the lower has 14 places
+            s = ((unsigned long long)(uint32_t)d[0] << 17) + (unsigned long long)(uint32_t)(d[2] * 131072.f);
+            for (int off = lpr >> 1; off >= 4; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+            return s;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        if (c < cpl) s += row_terms16(q[c]);
     for (int off = lpr >> 1; off >= 1; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
     return s;
+}
+
+constexpr int kPickSteps = 2;
+constexpr int kLazyRows = 4;  // stale rows a lazy-pick warp refreshes at once
+__host__ __device__ __forceinline__ void pick_layout(int J, int tile, int& cpl, int& lpr, int& rpw) {
+    const int cpr = J >> 4;
+    // at most 32 lanes a row: a row of 64 pieces (J = 1024) takes 2 a lane at least
+    const int least = (cpr + 31) >> 5;
+    int tl = tile == 1 || tile == 2 ? tile : 4;
+    if (tl < least) tl = least;
+    cpl = cpr < tl ? cpr : tl;
+    // whole quads of lanes from J = 64 on (row_sum)
+    while (J >= 64 && cpr / cpl < 4) cpl >>= 1;
+    lpr = cpr / cpl;
+    rpw = 32 / lpr;
 }
 
 __device__ __forceinline__ void lex_min(unsigned long long& S, int32_t& u, unsigned long long oS,
@@ -473,24 +561,11 @@ __device__ void pick_finish(const PickArgs& a, Top2 t) {
 
 
 // Full pick: S_u of every row (stored in lb when lazy picks follow).  Each
-// lane sums up to `tile` (1, 2 or 4: the J-tile width, a schedule knob)
-// consecutive 16-byte pieces of a row (LPR lanes a row, 32 / LPR rows a warp
-// step) and a warp issues the loads of kPickSteps steps before summing any,
-// so every warp keeps several KB of the stream in flight.
-constexpr int kPickSteps = 2;
-constexpr int kLazyRows = 4;  // stale rows a lazy-pick warp refreshes at once
-__host__ __device__ __forceinline__ void pick_layout(int J, int tile, int& cpl, int& lpr, int& rpw) {
-    const int cpr = J >> 4;
-    // at most 32 lanes a row: a row of 64 pieces (J = 1024) takes 2 a lane at least
-    const int least = (cpr + 31) >> 5;
-    int tl = tile == 1 || tile == 2 ? tile : 4;
-    if (tl < least) tl = least;
-    cpl = cpr < tl ? cpr : tl;
-    lpr = cpr / cpl;
-    rpw = 32 / lpr;
-}
-
-__global__ void __launch_bounds__(kBlock) k_pick(PickArgs a) {
+// lane takes up to `tile` (1, 2 or 4: the J-tile width, a schedule knob)
+// 16-byte pieces of a row (LPR lanes a row, 32 / LPR rows a warp step), and a
+// warp issues the loads of kPickSteps steps before summing any, so every warp
+// keeps several KB of the stream in flight.
+__global__ void __launch_bounds__(kBlock, 4) k_pick(PickArgs a) {
     const int J = a.J;
     int cpl, lpr, rpw;
     pick_layout(J, a.tile, cpl, lpr, rpw);
@@ -503,25 +578,16 @@ __global__ void __launch_bounds__(kBlock) k_pick(PickArgs a) {
     for (int64_t r0 = warp * step_rows; r0 < a.n; r0 += nwarps * step_rows) {
         uint4 q[kPickSteps][4];
 #pragma unroll
-        for (int u = 0; u < kPickSteps; ++u) {
-            const int64_t row = r0 + (int64_t)u * rpw + seg;
-            const uint4* p = reinterpret_cast<const uint4*>(a.M + (size_t)(row < a.n ? row : 0) * J) +
-                             seg_lane * cpl;
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                q[u][c] = (c < cpl && row < a.n) ? __ldcs(p + c) : make_uint4(0u, 0u, 0u, 0u);
-        }
+        for (int u = 0; u < kPickSteps; ++u)
+            load_row_pieces(a.M, J, r0 + (int64_t)u * rpw + seg, a.n, cpl, lpr, seg_lane, q[u]);
 #pragma unroll
         for (int u = 0; u < kPickSteps; ++u) {
             const int64_t row = r0 + (int64_t)u * rpw + seg;
-            unsigned long long sum = 0;
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (c < cpl) sum += row_terms16(q[u][c]);
-            for (int off = lpr >> 1; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+            const unsigned long long sum = row_sum(q[u], J, cpl, lpr);
             if (row < a.n && seg_lane == 0) {
                 if (a.lb) a.lb[row] = sum;
-                if (!is_picked(a.seed_bits, row)) t.insert(sum, (int32_t)row);
+                // (the seed bit's load waits only for a row that would be kept)
+                if (sum <= t.s2 && !is_picked(a.seed_bits, row)) t.insert(sum, (int32_t)row);
             }
         }
     }
@@ -725,21 +791,26 @@ cudaError_t launch_cover_seed(uint8_t* M, int J, int32_t s, const int32_t* rp_ou
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(kBlock) k_sums(const uint8_t* __restrict__ M, int32_t n, int J,
+__global__ void __launch_bounds__(kBlock, 4) k_sums(const uint8_t* __restrict__ M, int32_t n, int J,
                                                  unsigned long long* __restrict__ S) {
-    const int cpr = J >> 4;
-    const int lpr = cpr < 32 ? cpr : 32;
-    const int cpl = cpr / lpr;
-    const int rpw = 32 / lpr;
+    int cpl, lpr, rpw;
+    pick_layout(J, 4, cpl, lpr, rpw);
     const int lane = (int)lane_id();
     const int seg = lane / lpr, seg_lane = lane % lpr;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r0 = warp * rpw; r0 < n; r0 += nwarps * rpw) {
-        const int64_t row = r0 + seg;
-        const bool ok = row < n;
-        const unsigned long long s = row_sum(M, J, ok ? (int32_t)row : 0, lpr, cpl, seg_lane);
-        if (ok && seg_lane == 0) S[row] = s;
+    const int64_t step_rows = (int64_t)rpw * kPickSteps;
+    for (int64_t r0 = warp * step_rows; r0 < n; r0 += nwarps * step_rows) {
+        uint4 q[kPickSteps][4];
+#pragma unroll
+        for (int u = 0; u < kPickSteps; ++u)
+            load_row_pieces(M, J, r0 + (int64_t)u * rpw + seg, n, cpl, lpr, seg_lane, q[u]);
+#pragma unroll
+        for (int u = 0; u < kPickSteps; ++u) {
+            const int64_t row = r0 + (int64_t)u * rpw + seg;
+            const unsigned long long s = row_sum(q[u], J, cpl, lpr);
+            if (row < n && seg_lane == 0) S[row] = s;
+        }
     }
 }
 
@@ -1621,14 +1692,12 @@ namespace im {
 // its tiles, records the seed and its estimate, marks its row visited (the
 // graph's visited counter), and appends it to the cover's level-0 queue.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kBlock) k_batch_tiles(BatchPickArgs a) {
+__global__ void __launch_bounds__(kBlock, 4) k_batch_tiles(BatchPickArgs a) {
     __shared__ unsigned long long sS[kWarpsPerBlock];
     __shared__ int32_t sU[kWarpsPerBlock];
     const int J = a.J;
-    const int cpr = J >> 4;
-    const int lpr = cpr < 32 ? cpr : 32;
-    const int cpl = cpr / lpr;
-    const int rpw = 32 / lpr;
+    int cpl, lpr, rpw;
+    pick_layout(J, 4, cpl, lpr, rpw);
     const int lane = (int)lane_id();
     const int seg = lane / lpr, seg_lane = lane % lpr;
     const int wib = threadIdx.x >> 5;
@@ -1637,13 +1706,20 @@ __global__ void __launch_bounds__(kBlock) k_batch_tiles(BatchPickArgs a) {
         unsigned long long bestS = ~0ull;
         int32_t bestU = 0x7FFFFFFF;
         if (a.active[T.x]) {
-            for (int64_t r0 = (int64_t)T.y + (int64_t)wib * rpw; r0 < T.z; r0 += (int64_t)kWarpsPerBlock * rpw) {
-                const int64_t row = r0 + seg;
-                const bool ok = row < T.z;
-                const unsigned long long s = row_sum(a.M, J, ok ? (int32_t)row : T.y, lpr, cpl, seg_lane);
-                if (ok && seg_lane == 0) {
-                    const bool picked = (__ldcg(a.picked + (row >> 5)) >> (row & 31)) & 1u;
-                    if (!picked) lex_min(bestS, bestU, s, (int32_t)row);
+            const int64_t step_rows = (int64_t)rpw * kPickSteps;
+            for (int64_t r0 = (int64_t)T.y + wib * step_rows; r0 < T.z; r0 += kWarpsPerBlock * step_rows) {
+                uint4 q[kPickSteps][4];
+#pragma unroll
+                for (int u = 0; u < kPickSteps; ++u)
+                    load_row_pieces(a.M, J, r0 + (int64_t)u * rpw + seg, T.z, cpl, lpr, seg_lane, q[u]);
+#pragma unroll
+                for (int u = 0; u < kPickSteps; ++u) {
+                    const int64_t row = r0 + (int64_t)u * rpw + seg;
+                    const unsigned long long s = row_sum(q[u], J, cpl, lpr);
+                    // (the picked bit's load waits only for a row that would be kept)
+                    if (row < T.z && seg_lane == 0 && s <= bestS &&
+                        !((__ldcg(a.picked + (row >> 5)) >> (row & 31)) & 1u))
+                        lex_min(bestS, bestU, s, (int32_t)row);
                 }
             }
         }
