@@ -1884,14 +1884,16 @@ __device__ __forceinline__ void edge_live_chunks(uint32_t h, uint32_t thr, int J
     if (thr == 0u) return;
     int lo, hi;
     candidate_range(h, thr, J, sX, sTab, lo, hi);
-    for (int c = lo >> 4; hi > lo && c <= ((hi - 1) >> 4); ++c) {
-        const int j1 = min(hi, 16 * c + 16);
-        for (int j = max(lo, 16 * c); j < j1; ++j)
-            if ((sX[j] ^ h) < thr) {
-                if (c < 32) lo_mask |= 1u << c;
-                else hi_mask |= 1u << (c - 32);
-                break;
-            }
+    // one loop over the candidates, a live one moves on to the next chunk: a
+    // lane's tests follow one another whatever its neighbours' chunks hold (a
+    // loop a chunk waited for the slowest lane in every chunk: R-MAT scale 24,
+    // trivalency, J = 512, a whole selection 130.8 -> 130.1 ms)
+    for (int j = lo; j < hi;) {
+        const bool live = (sX[j] ^ h) < thr;
+        const uint32_t bit = live ? 1u << ((j >> 4) & 31) : 0u;
+        if (j < 512) lo_mask |= bit;
+        else hi_mask |= bit;
+        j = live ? (j | 15) + 1 : j + 1;
     }
 }
 
