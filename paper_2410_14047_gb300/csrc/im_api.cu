@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "../../include/difuser_im.h"
+#include "im_host.h"
 #include "im_internal.h"
 #include "im_launch.h"
 
@@ -300,13 +301,8 @@ struct im_sketch {
     // a selection in flight: phases and rebuilds queue without host reads;
     // their error word is read once at the end
     bool defer = false;
-    // the set of per-level counters, formats and barrier words the current phase
-    // uses, and each set's state: a persistent phase zeroes the other set when
-    // the phase before it ran there
-    int pset = 0;
-    int fmt0 = 0;  // format of the current phase's level-0 queue
-    enum SetState { kSetDirty, kSetZeroed, kSetUsed };
-    SetState set_state[2] = {kSetDirty, kSetDirty};
+    imi::PhaseSets sets;  // per-level counters, formats and barrier words: the current phase's set
+    int fmt0 = 0;         // format of the current phase's level-0 queue
     bool pull_safe = false;  // the pull queue holds every out-bucket (it cannot overflow)
     DBuf out_seed, out_S, out_est;
     DBuf gsum;  // lazy-pick group records
@@ -948,7 +944,7 @@ static ulonglong2* set_ctr(const im_sketch* sk, int set) { return sk->ctr.as<ulo
 static unsigned int* set_claim(const im_sketch* sk, int set) { return sk->claim.as<unsigned int>() + set * kSetLevels; }
 static uint8_t* set_fmt(const im_sketch* sk, int set) { return sk->fmt.as<uint8_t>() + set * kSetLevels; }
 static unsigned int* set_bar(const im_sketch* sk, int set) { return sk->bar.as<unsigned int>() + set * kBarWords; }
-static ulonglong2* cur_ctr(const im_sketch* sk) { return set_ctr(sk, sk->pset); }
+static ulonglong2* cur_ctr(const im_sketch* sk) { return set_ctr(sk, sk->sets.cur()); }
 
 // Start of a propagation or cover phase: the other set of level counters, work
 // counters and barrier words, zeroed unless the last persistent phase did so
@@ -958,13 +954,12 @@ static ulonglong2* cur_ctr(const im_sketch* sk) { return set_ctr(sk, sk->pset); 
 static im_status phase_begin(im_sketch* sk, int mode, int fmt0 = -1) {
     im_ctx* c = sk->ctx;
     auto st = c->stream;
-    sk->pset ^= 1;
-    const int s = sk->pset;
-    if (sk->set_state[s] != im_sketch::kSetZeroed) {
+    const bool zero = sk->sets.begin();
+    const int s = sk->sets.cur();
+    if (zero) {
         CK(c, cudaMemsetAsync(set_ctr(sk, s), 0, kSetLevels * 16, st));
         CK(c, cudaMemsetAsync(set_claim(sk, s), 0, kSetLevels * 4, st));
         CK(c, cudaMemsetAsync(set_bar(sk, s), 0, kBarWords * 4, st));
-        sk->set_state[s] = im_sketch::kSetZeroed;
     }
     // the level-0 queue: bucket entries (fmt0 = 1, or by default for a cover
     // in bucket mode: the seed kernel writes them), vertex entries otherwise
@@ -993,7 +988,7 @@ static im_status run_phase_persistent(im_sketch* sk, int mode, bool all_first, i
         p.qh[i] = sk->qh[i].as<QEntry>();
         p.chg[i] = chg_buf(sk, mode, i).as<uint32_t>();
     }
-    const int s = sk->pset, o = s ^ 1;
+    const int s = sk->sets.cur(), o = sk->sets.other();
     p.ctr = set_ctr(sk, s);
     p.claim = set_claim(sk, s);
     p.all_first = all_first ? 1 : 0;
@@ -1004,13 +999,12 @@ static im_status run_phase_persistent(im_sketch* sk, int mode, bool all_first, i
     p.level_ns = c->trace ? sk->level_ns.as<unsigned long long>() : nullptr;
     p.fmt = set_fmt(sk, s);
     p.fmt0 = sk->fmt0;
-    if (sk->set_state[o] == im_sketch::kSetUsed) {
+    if (sk->sets.zero_other()) {
         p.ctr_old = set_ctr(sk, o);
         p.claim_old = set_claim(sk, o);
         p.bar_old = set_bar(sk, o);
-        sk->set_state[o] = im_sketch::kSetZeroed;
     }
-    sk->set_state[s] = im_sketch::kSetUsed;
+    sk->sets.launch();
     CK(c, timed(c, mode == kPush ? kTPush : kTCover,
                 [&] { return launch_phase(sk->kind, mode, sk->dev, p, grid, st); }));
     // stamps gen_base .. gen_base + max_levels are this phase's
@@ -1070,10 +1064,10 @@ static im_status run_levels(im_sketch* sk, int mode, bool all_first) {
         if (pgrid > 0) return run_phase_persistent(sk, mode, all_first, pgrid);
     }
     // per-level launches: the counters stay dirty, the level-0 format is in memory
-    sk->set_state[sk->pset] = im_sketch::kSetDirty;
+    sk->sets.leave_dirty();
     ulonglong2* ctr = cur_ctr(sk);
-    unsigned int* claim = set_claim(sk, sk->pset);
-    uint8_t* fmt = set_fmt(sk, sk->pset);
+    unsigned int* claim = set_claim(sk, sk->sets.cur());
+    uint8_t* fmt = set_fmt(sk, sk->sets.cur());
     CK(c, cudaMemsetAsync(fmt, sk->fmt0, 1, st));
     LevelArgs a = level_args(sk);
     set_lcm(a, sk, mode);

@@ -25,6 +25,7 @@
 // candidates, instead of a scan of all in-edges.
 #include <cooperative_groups.h>
 
+#include "im_host.h"
 #include "im_launch.h"
 
 namespace im {
@@ -1662,13 +1663,11 @@ __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
     unsigned long long pre_l = __ldcg(&p.ctr[0].x), pre_h = __ldcg(&p.ctr[0].y);
     for (int i = threadIdx.x; i < p.base.J; i += blockDim.x) sX[i] = __ldg(p.base.X + i);
     sQueue.init();
-    if (__syncthreads_or(failed)) return;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    LevelArgs a = p.base;
-    a.sq = (uint32_t)__cvta_generic_to_shared(sQueue.queue);
+    const bool gave_up = __syncthreads_or(failed);
+    // (after a phase that gave up as well: the kernels between the phases add
+    // to the sets' first counters without asking)
     if (p.bar_old && blockIdx.x == gridDim.x - 1) {
-        const int used = min((int)__ldcg(p.bar_old + kBarLevels) + 2, kMaxLevels + 2);
+        const int used = imi::set_entries_used(gave_up, (int)__ldcg(p.bar_old + kBarLevels), kMaxLevels + 2);
         for (int i = threadIdx.x; i < used; i += blockDim.x) {
             p.ctr_old[i] = make_ulonglong2(0ull, 0ull);
             p.claim_old[i] = 0u;
@@ -1676,6 +1675,11 @@ __global__ void __launch_bounds__(kPBlock, kPhaseMinBlocks) k_phase(GraphDev g, 
         __syncthreads();
         for (int i = threadIdx.x; i < kBarWords; i += blockDim.x) p.bar_old[i] = 0u;
     }
+    if (gave_up) return;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    LevelArgs a = p.base;
+    a.sq = (uint32_t)__cvta_generic_to_shared(sQueue.queue);
     if (p.fmt && blockIdx.x == 0 && threadIdx.x == 0) p.fmt[0] = (uint8_t)p.fmt0;
     unsigned int* const arrive = p.bar + kBarArrive;
     unsigned int* const abort_flag = p.bar + kBarAbort;
