@@ -1004,9 +1004,10 @@ static im_status run_phase_persistent(im_sketch* sk, int mode, bool all_first, i
         p.claim_old = set_claim(sk, o);
         p.bar_old = set_bar(sk, o);
     }
-    sk->sets.launch();
+    sk->chg_dirty = true;  // until the phase is known to be queued (a selection) or to have ended well
     CK(c, timed(c, mode == kPush ? kTPush : kTCover,
                 [&] { return launch_phase(sk->kind, mode, sk->dev, p, grid, st); }));
+    sk->sets.launched();
     // stamps gen_base .. gen_base + max_levels are this phase's
     sk->gen_counter += kMaxLevels;
     if (sk->gen_counter > (1 << 30)) {
@@ -1020,7 +1021,6 @@ static im_status run_phase_persistent(im_sketch* sk, int mode, bool all_first, i
     CK(c, cudaMemcpyAsync(c->pinned, p.bar + kBarLevels, 4, cudaMemcpyDeviceToHost, st));
     CK(c, sync_collect(c));
     const int levels = *reinterpret_cast<const int*>(c->pinned);
-    sk->chg_dirty = true;
     if (c->trace && levels > 0 && levels < p.max_levels) {
         // per-level records from the in-kernel clock (one launch for all levels)
         std::vector<ulonglong2> h((size_t)levels);
@@ -1063,8 +1063,7 @@ static im_status run_levels(im_sketch* sk, int mode, bool all_first) {
         const int pgrid = phase_blocks(c, phase_grid());
         if (pgrid > 0) return run_phase_persistent(sk, mode, all_first, pgrid);
     }
-    // per-level launches: the counters stay dirty, the level-0 format is in memory
-    sk->sets.leave_dirty();
+    // per-level launches: the set stays dirty, the level-0 format is in memory
     ulonglong2* ctr = cur_ctr(sk);
     unsigned int* claim = set_claim(sk, sk->sets.cur());
     uint8_t* fmt = set_fmt(sk, sk->sets.cur());

@@ -23,7 +23,8 @@ IM_HD int set_entries_used(bool gave_up, int levels, int all) {
 // phases of a sketch use in turn.  A set has to be zero when its phase begins
 // (level 0 is written by the kernels before the phase's launch): the phase
 // launch in between zeroes what the one before it used, otherwise the host
-// zeroes all of it.
+// zeroes all of it (after a phase that ran in launches of their own, or whose
+// launch failed: then nothing ran).
 class PhaseSets {
 public:
     int cur() const { return cur_; }
@@ -32,18 +33,16 @@ public:
     bool begin() {
         cur_ ^= 1;
         const bool zero = state_[cur_] != kZeroed;
-        state_[cur_] = kZeroed;
+        state_[cur_] = kDirty;
         return zero;
     }
-    // Its launch zeroes what the phase before it used in the other set.
+    // Its launch is to zero what the phase before it used in the other set.
     bool zero_other() const { return state_[other()] == kUsed; }
-    // That launch comes.
-    void launch() {
+    // That launch went out.
+    void launched() {
         if (zero_other()) state_[other()] = kZeroed;
         state_[cur_] = kUsed;
     }
-    // The phase runs in launches that zero nothing.
-    void leave_dirty() { state_[cur_] = kDirty; }
 
 private:
     enum State { kDirty, kZeroed, kUsed };

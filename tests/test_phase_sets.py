@@ -43,13 +43,11 @@ int main(int argc, char** argv) {
             const int what = rand() % 10;
             if (what == 0 && (kinds & 2)) {  // a launch a level
                 for (int l = 0; l < 5; ++l) d.ctr[s][l] = 1;
-                sets.leave_dirty();
                 continue;
             }
-            // LAUNCH
             const bool zero_other = sets.zero_other();
             if (what == 1 && (kinds & 4)) continue;  // the launch fails: nothing ran
-            sets.launch();
+            sets.launched();
             const bool before = d.gave_up;
             if (what == 2 && (kinds & 1)) d.gave_up = true;
             // a block that starts late may find this launch's own give-up
@@ -91,6 +89,6 @@ def _run(tmp_path, kinds):
     assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout
 
 
-@pytest.mark.parametrize("kinds", [0, 1, 2, 3], ids=["complete", "give_up", "per_level", "both"])
+@pytest.mark.parametrize("kinds", [0, 1, 2, 4, 7], ids=["complete", "give_up", "per_level", "launch_fails", "all"])
 def test_a_set_is_zero_when_its_phase_begins(tmp_path, kinds):
     _run(tmp_path, kinds)
