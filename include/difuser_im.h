@@ -401,7 +401,13 @@ IM_API im_status im_fill_rate(im_graph* g, int32_t J, uint64_t seed, const im_mo
  * `slots` worker threads, each with its own CUDA stream and stream-ordered
  * memory pool, so the kernels of up to `slots` queries overlap on the device
  * (continuous batching: a query starts as soon as a slot and its device memory
- * are free, while others are running).  Admission control: the resident graphs
+ * are free, while others are running).  The phases of all calls that run on a
+ * device at the same time (every server's queries and every context's own
+ * selections, builds, covers, rebuilds and batches in the process) divide its
+ * blocks evenly, since the blocks of a phase wait for one another between its
+ * levels: a call waits at its first phase, holding its device memory, until the
+ * others have come down to the new share, a selection at its next seed, a batch
+ * at its next round, a step-level call at its end.  Admission control: the resident graphs
  * plus the device bytes reserved by running queries (im_server_query_bytes,
  * an exact upper bound of what a query allocates) never exceed the budget.
  * Pending queries start in arrival order; one that fits may start ahead of an

@@ -33,8 +33,8 @@ struct im_ctx {
     uint64_t peak = 0;
     bool custom_alloc = false;
     im_allocator alloc{};
-    imi::BlockShares* shares = nullptr;  // a server's worker: where its launches' blocks come from
-    int blocks = 0;                      // held of them by the query that runs
+    imi::BlockAccount* account = nullptr;  // the device's blocks, while a call that runs phases does (PhaseCall)
+    int blocks = 0;                        // held of them by that call
     cudaMemPool_t pool = nullptr;  // stream-ordered pool of a server worker (else the device default)
     std::unordered_map<void*, size_t> sizes;
     std::string err;
@@ -318,6 +318,37 @@ struct im_sketch {
     const int32_t* gid = nullptr;
     unsigned long long* gcount = nullptr;
     const uint8_t* gflag = nullptr;
+};
+
+// One call that runs phases: its part of the device's blocks (BlockAccount),
+// taken at its first phase and returned at its end.  Without cooperative
+// launches (tuning.persistent 0) no block waits for another, and it takes none.
+struct PhaseCall {
+    im_ctx* c;
+    bool idle = false;  // set when everything the call queued has completed
+    explicit PhaseCall(im_ctx* ctx) : c(ctx) {
+        const int resident = c->tuning.persistent ? imi::resident_blocks() : 0;
+        if (resident <= 0) return;
+        c->account = imi::account_of(c->device, resident);
+        c->account->enter();
+    }
+    PhaseCall(const PhaseCall&) = delete;
+    // Nothing of this call is in flight: blocks for others, or more for it.
+    void adjust() {
+        if (c->account && c->blocks > 0) c->blocks = c->account->adjust(c->blocks);
+    }
+    im_status done(im_status s) {
+        idle = s == IM_OK;
+        return s;
+    }
+    ~PhaseCall() {
+        if (!c->account) return;
+        // a failed call may have a phase in flight
+        if (!idle && c->blocks > 0) cudaStreamSynchronize(c->stream);
+        c->account->leave(c->blocks);
+        c->blocks = 0;
+        c->account = nullptr;
+    }
 };
 
 // ---------------------------------------------------------------------------
@@ -1045,12 +1076,6 @@ static im_status run_phase_persistent(im_sketch* sk, int mode, bool all_first, i
     return IM_OK;
 }
 
-// Blocks of a phase launch: every resident block (at most 2048), or a query's
-// share of them in a server.
-static int phase_blocks(const im_ctx* c, int grid) {
-    return std::min(grid, c->shares ? c->blocks : 64 * 32);
-}
-
 // Runs frontier levels until both queues are empty.  Level t reads queue
 // t % 3 with counters ctr[t], writes queue (t+1) % 3 with counters ctr[t+1],
 // and clears the change bits of queue (t+2) % 3 (read by level t-1).  The host
@@ -1059,9 +1084,9 @@ static int phase_blocks(const im_ctx* c, int grid) {
 static im_status run_levels(im_sketch* sk, int mode, bool all_first) {
     im_ctx* c = sk->ctx;
     auto st = c->stream;
-    if (c->tuning.persistent) {
-        const int pgrid = phase_blocks(c, phase_grid());
-        if (pgrid > 0) return run_phase_persistent(sk, mode, all_first, pgrid);
+    if (c->account) {
+        if (c->blocks == 0) c->blocks = c->account->take();
+        return run_phase_persistent(sk, mode, all_first, c->blocks);
     }
     // per-level launches: the set stays dirty, the level-0 format is in memory
     ulonglong2* ctr = cur_ctr(sk);
@@ -1493,10 +1518,11 @@ extern "C" im_status im_sketch_build(im_graph* g, int32_t J, uint64_t seed, im_s
     im_ctx* c = g->ctx;
     stats_begin(c);
     const double t0 = now_ms();
+    PhaseCall call(c);
     im_sketch* sk = nullptr;
     CKS(sketch_start(c, g, J, seed, nullptr, true, &sk));
     im_status s = build_registers(sk);
-    if (s == IM_OK) s = stats_collect(sk);
+    if (s == IM_OK) s = call.done(stats_collect(sk));
     if (s != IM_OK) {
         sketch_release(sk);
         delete sk;
@@ -1643,12 +1669,13 @@ extern "C" im_status im_sketch_cover(im_sketch* sk, int32_t s, uint64_t* count_o
     if (!sk) return IM_E_INVAL;
     im_ctx* c = sk->ctx;
     if (s < 0 || s >= sk->g->n) return fail(c, IM_E_RANGE, "vertex %d out of range", s);
+    PhaseCall call(c);
     CKS(phase_begin(sk, kCover));
     CK(c, launch_cover_seed(sk->M.as<uint8_t>(), sk->J, s, sk->g->rp_out.as<int32_t>(),
                             sk->ql[0].as<QEntry>(), &cur_ctr(sk)[0].x,
                             chg_buf(sk, kCover, 0).as<uint32_t>(), sk->count.as<unsigned long long>(),
                             sk->buckets ? sk->bk_end[1].as<uint32_t>() : nullptr, sk->J / 16, c->stream));
-    CKS(run_levels(sk, kCover, false));
+    CKS(call.done(run_levels(sk, kCover, false)));
     if (count_out) {
         unsigned long long cnt = 0;
         CK(c, cudaMemcpyAsync(&cnt, sk->count.p, 8, cudaMemcpyDeviceToHost, c->stream));
@@ -1660,7 +1687,8 @@ extern "C" im_status im_sketch_cover(im_sketch* sk, int32_t s, uint64_t* count_o
 
 extern "C" im_status im_sketch_rebuild(im_sketch* sk) {
     if (!sk) return IM_E_INVAL;
-    return build_registers(sk);
+    PhaseCall call(sk->ctx);
+    return call.done(build_registers(sk));
 }
 
 // ---------------------------------------------------------------------------
@@ -1682,6 +1710,7 @@ static im_status select_seeds_impl(im_ctx* c, im_graph* g, int32_t K, int32_t J,
     }
     stats_begin(c);
     const double t0 = now_ms();
+    PhaseCall call(c);
     im_sketch* sk = nullptr;
     CKS(sketch_start(c, g, J, seed, model, true, &sk));
     sk->lazy = c->tuning.lazy_pick != 0;
@@ -1696,7 +1725,6 @@ static im_status select_seeds_impl(im_ctx* c, im_graph* g, int32_t K, int32_t J,
     };
     im_status s = ensure_out_cap(sk, K);
     if (s != IM_OK) return bail(s);
-    if (c->shares) c->blocks = c->shares->take();
     if ((s = build_registers(sk)) != IM_OK) return bail(s);
     const double t_build = now_ms();
     c->stats.ms_build = t_build - t0;
@@ -1711,7 +1739,7 @@ static im_status select_seeds_impl(im_ctx* c, im_graph* g, int32_t K, int32_t J,
         if (e == cudaSuccess) e = sync_collect(c);
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "read count"));
         const uint64_t count = c->pinned[0];
-        if (c->shares) c->blocks = c->shares->adjust(c->blocks);  // (nothing of this query is in flight)
+        call.adjust();
         score[k] = (double)count / (double)J;
         const double tr = now_ms();
         ms_pc += tr - tk;
@@ -1733,7 +1761,7 @@ static im_status select_seeds_impl(im_ctx* c, im_graph* g, int32_t K, int32_t J,
         e = cudaMemcpyAsync(est.data(), sk->out_est.p, (size_t)K * 8, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "read seeds"));
-    if ((s = stats_collect(sk)) != IM_OK) return bail(s);
+    if ((s = call.done(stats_collect(sk))) != IM_OK) return bail(s);
     c->stats.builds = 1 + rebuilds;
     c->stats.ms_rebuild = ms_rebuild;
     c->stats.ms_pick = ms_pc;
@@ -1802,12 +1830,11 @@ namespace imi {
 
 int resident_blocks() { return std::min(phase_grid(), 64 * 32); }
 
-im_status ctx_create_worker(int device, cudaStream_t stream, cudaMemPool_t pool, BlockShares* shares, im_ctx** out) {
+im_status ctx_create_worker(int device, cudaStream_t stream, cudaMemPool_t pool, bool persistent, im_ctx** out) {
     im_ctx* c = nullptr;
     CKS(im_ctx_create(device, stream, 0, nullptr, &c));
     c->pool = pool;
-    c->shares = shares;
-    c->tuning.persistent = shares ? 1 : 0;
+    c->tuning.persistent = persistent ? 1 : 0;
     *out = c;
     return IM_OK;
 }
@@ -1818,16 +1845,7 @@ const char* ctx_error(const im_ctx* c) { return c->err.c_str(); }
 im_status select_seeds_on(im_ctx* c, im_graph* g, int32_t K, int32_t J, const im_model* model,
                           uint64_t seed, double rebuild_eps, int32_t* seeds_out, double* score_out,
                           double* estimate_out) {
-    if (c->shares) c->shares->enter();
-    const im_status s = select_seeds_impl(c, g, K, J, model, seed, rebuild_eps, seeds_out, score_out, estimate_out,
-                                          nullptr);
-    if (c->shares) {
-        // a failed query may have phases in flight
-        if (s != IM_OK) cudaStreamSynchronize(c->stream);
-        c->shares->leave(c->blocks);
-        c->blocks = 0;
-    }
-    return s;
+    return select_seeds_impl(c, g, K, J, model, seed, rebuild_eps, seeds_out, score_out, estimate_out, nullptr);
 }
 
 uint64_t query_bytes(const im_graph* g, int32_t J, int32_t K) {
@@ -2094,6 +2112,7 @@ extern "C" im_status im_batch_select_seeds(im_batch* b, const int32_t* J, const 
     }
     stats_begin(c);
     const double t0 = now_ms();
+    PhaseCall call(c);
     auto st = c->stream;
     std::vector<int32_t> Js(J, J + G);
     std::sort(Js.begin(), Js.end());
@@ -2188,6 +2207,7 @@ extern "C" im_status im_batch_select_seeds(im_batch* b, const int32_t* J, const 
             e = cudaMemcpyAsync(count.data(), gcount_d.p, (size_t)G * 8, cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = sync_collect(c);
             if (e != cudaSuccess) { cleanup(); return cuda_fail(c, e, "batch counts"); }
+            call.adjust();
             bool any = false;
             for (int32_t g : members) {
                 flag[g] = 0;
@@ -2224,6 +2244,7 @@ extern "C" im_status im_batch_select_seeds(im_batch* b, const int32_t* J, const 
         if ((s = stats_collect(sk)) != IM_OK) { cleanup(); return s; }
         cleanup();
     }
+    call.done(IM_OK);
     c->stats.builds = builds;
     c->stats.ms_total = now_ms() - t0;
     return IM_OK;

@@ -1,7 +1,10 @@
 // Host-side bookkeeping that needs no CUDA (compiled and tested on the CPU as
-// well): which counter set a phase runs on.
+// well): which counter set a phase runs on, and how the calls that run at the
+// same time divide a device's blocks.
 #pragma once
-#include <algorithm>
+#include <condition_variable>
+#include <map>
+#include <mutex>
 
 #ifdef __CUDACC__
 #define IM_HD __host__ __device__ __forceinline__
@@ -49,5 +52,68 @@ private:
     int cur_ = 0;
     State state_[2] = {kDirty, kDirty};
 };
+
+// The blocks of one device that fit it at once in every phase launch, divided
+// among the calls that run phases.  A phase runs all its levels in one
+// cooperative launch whose blocks wait for one another, so the grids in flight
+// must never add up to more than the device holds: a call takes blocks before
+// its first phase, gives back or takes more only while none of its phases is in
+// flight, and returns them at its end.  The even share is total / running: a
+// call that joins waits until the others have come down to it, a selection at
+// its next seed.
+class BlockAccount {
+public:
+    explicit BlockAccount(int total) : total_(total), free_(total) {}
+    int total() const { return total_; }
+
+    // A call starts; leave ends it and returns what it holds.
+    void enter() {
+        std::lock_guard<std::mutex> lk(mu_);
+        ++running_;
+    }
+    void leave(int held) {
+        std::lock_guard<std::mutex> lk(mu_);
+        --running_;
+        free_ += held;
+        cv_.notify_all();
+    }
+    // Its first phase comes: waits for its share, returns it.
+    int take() {
+        std::unique_lock<std::mutex> lk(mu_);
+        cv_.wait(lk, [&] { return free_ >= even(); });
+        const int take = even();
+        free_ -= take;
+        return take;
+    }
+    // No phase of it is in flight: its new share in place of `held`.
+    int adjust(int held) {
+        std::lock_guard<std::mutex> lk(mu_);
+        const int want = even(), most = held + free_;
+        const int take = want < most ? want : most;
+        free_ += held - take;
+        if (take < held) cv_.notify_all();
+        return take;
+    }
+
+private:
+    int even() const { return total_ > running_ ? total_ / running_ : 1; }
+    std::mutex mu_;
+    std::condition_variable cv_;
+    const int total_;
+    int free_;
+    int running_ = 0;
+};
+
+// The device's account: one for the whole process, from which every server's
+// queries and every context's calls take (`total`: the device's blocks, the
+// same at each call).  It lives until the process ends.
+inline BlockAccount* account_of(int device, int total) {
+    static std::mutex mu;
+    static auto* accounts = new std::map<int, BlockAccount*>;
+    std::lock_guard<std::mutex> lk(mu);
+    BlockAccount*& a = (*accounts)[device];
+    if (!a) a = new BlockAccount(total);
+    return a;
+}
 
 }  // namespace imi

@@ -2,48 +2,19 @@
 // library (hidden symbols: not part of the C ABI).
 #pragma once
 #include <cuda_runtime.h>
-#include <condition_variable>
 #include <cstdint>
-#include <mutex>
 
 #include "../../include/difuser_im.h"
 
 namespace imi {
 
-// The resident blocks that the running queries of a server divide among them.
-// A phase runs all its levels in one cooperative launch whose blocks wait for
-// one another, so the grids in flight never add up to more than the GPU holds
-// at once: a query takes blocks before its first launch, gives back or takes
-// more only while none of its launches is in flight, and returns them at its
-// end.  The even share is total / running: a query that joins waits until the
-// others, at their next seed, have come down to it.
-class BlockShares {
-public:
-    explicit BlockShares(int total) : total_(total), free_(total) {}
-    // A query starts; leave ends it and returns what it holds.
-    void enter();
-    void leave(int held);
-    // Its first phase comes: waits for its share, returns it.
-    int take();
-    // No phase of it is in flight: its new share in place of `held`.
-    int adjust(int held);
-
-private:
-    int even() const { return total_ / running_ > 0 ? total_ / running_ : 1; }
-    std::mutex mu_;
-    std::condition_variable cv_;
-    const int total_;
-    int free_;
-    int running_ = 0;
-};
-
 // Blocks that fit the current device at once in every phase launch (0: no
 // cooperative launch).
 int resident_blocks();
 
-// A context that runs on `stream`, allocates from `pool` (stream-ordered) and
-// takes the grids of its phase launches from `shares` (NULL: a launch a level).
-im_status ctx_create_worker(int device, cudaStream_t stream, cudaMemPool_t pool, BlockShares* shares, im_ctx** out);
+// A context that runs on `stream` and allocates from `pool` (stream-ordered);
+// persistent 0: a launch a level.
+im_status ctx_create_worker(int device, cudaStream_t stream, cudaMemPool_t pool, bool persistent, im_ctx** out);
 void ctx_set_budget(im_ctx* c, uint64_t bytes);
 const char* ctx_error(const im_ctx* c);
 

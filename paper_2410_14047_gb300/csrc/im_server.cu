@@ -10,7 +10,6 @@
 #include <cstdio>
 #include <cstring>
 #include <deque>
-#include <memory>
 #include <mutex>
 #include <thread>
 #include <unordered_map>
@@ -18,40 +17,6 @@
 
 #include "../../include/difuser_im.h"
 #include "im_internal.h"
-
-namespace imi {
-
-void BlockShares::enter() {
-    std::lock_guard<std::mutex> lk(mu_);
-    ++running_;
-}
-
-int BlockShares::take() {
-    std::unique_lock<std::mutex> lk(mu_);
-    cv_.wait(lk, [&] { return free_ >= even(); });
-    const int take = even();
-    free_ -= take;
-    return take;
-}
-
-int BlockShares::adjust(int held) {
-    std::lock_guard<std::mutex> lk(mu_);
-    const int want = even(), most = held + free_;
-    const int take = want < most ? want : most;
-    if (take == held) return held;
-    free_ += held - take;
-    if (take < held) cv_.notify_all();
-    return take;
-}
-
-void BlockShares::leave(int held) {
-    std::lock_guard<std::mutex> lk(mu_);
-    --running_;
-    free_ += held;
-    cv_.notify_all();
-}
-
-}  // namespace imi
 
 namespace {
 
@@ -88,7 +53,6 @@ struct im_server {
     int64_t next_ticket = 1, submitted = 0, completed = 0, failed = 0, bypassed = 0;
     bool stop = false;
     cudaMemPool_t pool = nullptr;
-    std::unique_ptr<imi::BlockShares> shares;
     std::vector<cudaStream_t> streams;
     std::vector<im_ctx*> ctxs;
     std::vector<std::thread> workers;
@@ -191,14 +155,13 @@ extern "C" im_status im_server_create(const im_server_config* cfg, im_server** o
     uint64_t keep = UINT64_MAX;
     if (cudaMemPoolSetAttribute(srv->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess)
         return bail();
-    const int resident = imi::resident_blocks();
-    if (resident >= cfg->slots) srv->shares.reset(new imi::BlockShares(resident));
+    const bool persistent = imi::resident_blocks() >= cfg->slots;
     for (int i = 0; i < cfg->slots; ++i) {
         cudaStream_t st = nullptr;
         if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) return bail();
         srv->streams.push_back(st);
         im_ctx* c = nullptr;
-        if (imi::ctx_create_worker(cfg->device, st, srv->pool, srv->shares.get(), &c) != IM_OK) return bail();
+        if (imi::ctx_create_worker(cfg->device, st, srv->pool, persistent, &c) != IM_OK) return bail();
         srv->ctxs.push_back(c);
     }
     for (int i = 0; i < cfg->slots; ++i) srv->workers.emplace_back([srv, i] { srv->worker(i); });
