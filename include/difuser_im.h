@@ -227,7 +227,9 @@ IM_API im_status im_ctx_get_tuning(const im_ctx* ctx, im_tuning* tuning);
  * two levels of a phase (all levels of a build or a cover run in one
  * cooperative launch); a block that waits longer raises an abort word, every
  * block leaves the launch at its next barrier, and the call returns
- * IM_E_TIMEOUT (0: a block that has to wait at all gives up at once).
+ * IM_E_TIMEOUT (0: a block that has to wait at all gives up at once).  The
+ * value is for a call that holds all of the device's blocks: beside other
+ * calls (see the served form) a phase on 1/f of them waits f times as long.
  * max_levels bounds the levels of one phase (propagation to the fixpoint,
  * one cover, one affected-set search): a frontier still non-empty after
  * max_levels levels ends the phase with IM_E_TIMEOUT.  Defaults: 2 s and

@@ -1026,7 +1026,7 @@ static im_status run_phase_persistent(im_sketch* sk, int mode, bool all_first, i
     p.max_levels = c->max_levels;
     p.gen_base = sk->gen_counter + 1;
     p.bar = set_bar(sk, s);
-    p.limit_ns = c->barrier_limit_ns;
+    p.limit_ns = imi::wait_limit(c->barrier_limit_ns, c->account->total(), grid);
     p.level_ns = c->trace ? sk->level_ns.as<unsigned long long>() : nullptr;
     p.fmt = set_fmt(sk, s);
     p.fmt0 = sk->fmt0;

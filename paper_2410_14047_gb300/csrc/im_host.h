@@ -1,8 +1,9 @@
 // Host-side bookkeeping that needs no CUDA (compiled and tested on the CPU as
-// well): which counter set a phase runs on, and how the calls that run at the
-// same time divide a device's blocks.
+// well): which counter set a phase runs on, how the calls that run at the same
+// time divide a device's blocks, and how long a phase on some of them may wait.
 #pragma once
 #include <condition_variable>
+#include <cstdint>
 #include <map>
 #include <mutex>
 
@@ -103,6 +104,16 @@ private:
     int free_;
     int running_ = 0;
 };
+
+// The bound on a barrier wait of a phase on `blocks` of the device's `total`, from
+// the bound `ns` for all of them: a level's work is the same on fewer blocks, so
+// it and the wait for its slowest block take up to total / blocks times as long
+// (one of 40 queries holds 7 of 304 blocks).  0 (give up at the first poll)
+// stays 0.
+inline uint64_t wait_limit(uint64_t ns, int total, int blocks) {
+    const uint64_t times = blocks < total ? ((uint64_t)total + (uint64_t)blocks - 1) / (uint64_t)blocks : 1;
+    return ns > UINT64_MAX / times ? UINT64_MAX : ns * times;
+}
 
 // The device's account: one for the whole process, from which every server's
 // queries and every context's calls take (`total`: the device's blocks, the

@@ -1,7 +1,7 @@
 """The device's blocks divided among concurrent calls, on the CPU (im_host.h):
 two servers' queries and plain contexts' calls take from one account, so that
 what they hold together never exceeds the device, and every waiting call gets
-its share."""
+its share; and the wait limit of a phase on a share."""
 import os
 import subprocess
 
@@ -80,8 +80,30 @@ int main(int argc, char** argv) {
 
 @pytest.mark.parametrize("total,threads", [(304, 16), (304, 3), (7, 24), (2, 24)])
 def test_callers_of_a_device_never_hold_more_than_it_has(tmp_path, total, threads):
+    assert _run(tmp_path, PROGRAM, total, threads) == ["ok"]
+
+
+LIMITS = r"""
+#include <cstdio>
+#include "im_host.h"
+int main() {
+    const unsigned long long ns[] = {0, 1, 2000000000ull, ~0ull / 2, ~0ull};
+    for (unsigned long long n : ns)
+        for (int blocks : {304, 303, 152, 101, 7, 4, 1}) printf("%llu\n", (unsigned long long)imi::wait_limit(n, 304, blocks));
+}
+"""
+
+
+def test_wait_limit_grows_with_what_a_share_lacks(tmp_path):
+    got = iter(int(x) for x in _run(tmp_path, LIMITS))
+    for ns in (0, 1, 2 * 10**9, (2**64 - 1) // 2, 2**64 - 1):
+        for blocks in (304, 303, 152, 101, 7, 4, 1):
+            assert next(got) == min(2**64 - 1, ns * -(-304 // blocks)), (ns, blocks)
+
+
+def _run(tmp_path, program, *args):
     src = tmp_path / "account.cpp"
-    src.write_text(PROGRAM)
+    src.write_text(program)
     exe = tmp_path / "account"
     try:
         r = subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-I", CSRC, str(src), "-o", str(exe)],
@@ -89,5 +111,6 @@ def test_callers_of_a_device_never_hold_more_than_it_has(tmp_path, total, thread
     except FileNotFoundError:
         pytest.skip("no C++ compiler")
     assert r.returncode == 0, r.stderr[-2000:]
-    r = subprocess.run([str(exe), str(total), str(threads)], capture_output=True, text=True, timeout=60)
-    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout
+    r = subprocess.run([str(exe), *map(str, args)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout
+    return r.stdout.split()
