@@ -2195,6 +2195,7 @@ extern "C" im_status im_batch_select_seeds(im_batch* b, const int32_t* J, const 
             pa.out_est = oest.as<double>();
             pa.rp_out = b->g->rp_out.as<int32_t>();
             pa.q_cover = sk->ql[0].as<QEntry>();
+            pa.q_cap = sk->buckets ? sk->bq_cap : b->g->n;
             pa.ctr_cover = &cur_ctr(sk)[0].x;
             pa.chg0 = chg_buf(sk, kCover, 0).as<uint32_t>();
             pa.gcount = sk->gcount;

@@ -335,10 +335,12 @@ __device__ __forceinline__ SeedBuckets seed_bucket_bounds(int32_t s, int C, cons
 // Bucket mode: queues the seed's out-buckets whose chunk has newly visited
 // simulations (level 0 of its cover); a chunk without live out-edges keeps
 // no change bits.  One warp, its lanes a chunk each, bits = the seed's change
-// words.  (A single thread walked the chunks twice, a load after the other:
+// words.  Entries past the queue's capacity cap are counted only: the level
+// then walks every bucket.  (A single thread walked the chunks twice, a load after the other:
 // R-MAT scale 17, J = 1024, 64 chunks, K = 25 took 6.77 ms, and 6.59 ms this way.)
 __device__ __forceinline__ void cover_seed_buckets(int32_t s, const uint32_t* bits, const SeedBuckets& k,
-                                                   uint32_t* chg_row, int C, QEntry* q, unsigned long long* ctr) {
+                                                   uint32_t* chg_row, int C, QEntry* q, uint32_t cap,
+                                                   unsigned long long* ctr) {
     const int lane = (int)lane_id();
     uint16_t* h16 = reinterpret_cast<uint16_t*>(chg_row);
     bool want[2];
@@ -371,7 +373,8 @@ __device__ __forceinline__ void cover_seed_buckets(int32_t s, const uint32_t* bi
         QEntry e;
         e.v = (int32_t)((uint32_t)s * (uint32_t)C + (uint32_t)(lane + 32 * h));
         e.rp = (int32_t)k.st[h]; e.off = (int32_t)off; e.aux = len[h];
-        q[slot++] = e;
+        if (slot < cap) q[slot] = e;
+        ++slot;
         off += len[h];
     }
 }
@@ -428,7 +431,8 @@ __device__ void cover_seed_block(uint8_t* M, int J, int32_t s, const int32_t* rp
         }
     }
     __syncwarp();
-    if (bk_end && nw) cover_seed_buckets(s, bits, k, chg_row, C, q, ctr);
+    // (the queue holds the buckets of one vertex)
+    if (bk_end && nw) cover_seed_buckets(s, bits, k, chg_row, C, q, (uint32_t)C, ctr);
 }
 
 // Least and second-least (S, u) pairs in lexicographic order.
@@ -1821,12 +1825,12 @@ __global__ void __launch_bounds__(kBlock) k_batch_graphs(BatchPickArgs a) {
     if (wib != 0 || nw == 0u) return;
     if (lane == 0) atomicAdd(a.gcount + g, (unsigned long long)nw);
     if (a.bk_end_out) {
-        cover_seed_buckets(s, bits, k, chg_row, a.chunks, a.q_cover, a.ctr_cover);
+        cover_seed_buckets(s, bits, k, chg_row, a.chunks, a.q_cover, (uint32_t)a.q_cap, a.ctr_cover);
     } else if (lane == 0 && deg > 0) {
         const unsigned long long base = atomicAdd(a.ctr_cover, (1ull << kCountShift) | (unsigned long long)deg);
         QEntry e;
         e.v = s; e.rp = rp; e.off = (int32_t)(base & kEdgeMask); e.aux = 0;
-        a.q_cover[base >> kCountShift] = e;
+        a.q_cover[chk((int64_t)(base >> kCountShift), a.q_cap, a.err)] = e;
     }
 }
 

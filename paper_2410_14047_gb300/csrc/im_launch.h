@@ -271,6 +271,7 @@ struct BatchPickArgs {
     double* out_est;
     const int32_t* rp_out;
     QEntry* q_cover;              // cover level-0 queue
+    int32_t q_cap;                // its entries (a vertex queue holds every vertex)
     unsigned long long* ctr_cover;
     uint32_t* chg0;
     unsigned long long* gcount;
