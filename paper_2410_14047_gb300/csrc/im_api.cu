@@ -1410,7 +1410,7 @@ static im_status build_buckets(im_sketch* sk) {
             e = timed(c, kTOther, [&] {
                 return launch_buckets(0, sk->kind, o == 0 ? kPush : kCover, sk->dev, sk->X.as<uint32_t>(),
                                       lcm_lo[o], lcm_hi[o], J, sk->bk_end[o].as<uint32_t>(),
-                                      ne.as<unsigned long long>() + o, nullptr, nullptr, st);
+                                      ne.as<unsigned long long>() + o, nullptr, nullptr, 0, nullptr, st);
             });
     }
     int64_t total[2] = {0, 0};
@@ -1438,7 +1438,8 @@ static im_status build_buckets(im_sketch* sk) {
         e = timed(c, kTOther, [&] {
             return launch_buckets(1, sk->kind, o == 0 ? kPush : kCover, sk->dev, sk->X.as<uint32_t>(),
                                   lcm_lo[o], lcm_hi[o], J, sk->bk_end[o].as<uint32_t>(), nullptr,
-                                  sk->bk_other[o].as<int32_t>(), sk->bk_mask[o].as<uint16_t>(), st);
+                                  sk->bk_other[o].as<int32_t>(), sk->bk_mask[o].as<uint16_t>(), total[o],
+                                  sk->err.as<uint32_t>(), st);
         });
     if (e != cudaSuccess) { drop(); return cuda_fail(c, e, "bucket fill"); }
     dfree(c, tmp);
@@ -1926,13 +1927,13 @@ extern "C" im_status im_spread_mc(im_graph* g, const int32_t* seeds, int32_t k, 
     if (s == IM_OK) s = dalloc(c, (size_t)(kMaxLevels + 2) * 8, ctr);
     if (s == IM_OK) s = dalloc(c, (size_t)n * 4, gen);
     if (s == IM_OK) s = dalloc(c, (size_t)1024 * 8, reach);
-    if (s == IM_OK) s = dalloc(c, 16, acc);
+    if (s == IM_OK) s = dalloc(c, 24, acc);  // sum, sum of squares, error word
     if (s == IM_OK) s = dalloc(c, (size_t)k * 4, sd);
     if (s != IM_OK) { release(); return s; }
     auto st = c->stream;
     cudaError_t e = cudaMemcpyAsync(sd.p, seeds, (size_t)k * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(gen.p, 0, gen.bytes, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(acc.p, 0, 16, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(acc.p, 0, 24, st);
     if (e != cudaSuccess) { release(); return cuda_fail(c, e, "spread init"); }
     unsigned long long* cp = ctr.as<unsigned long long>();
     const int grid = mc_grid();
@@ -1951,6 +1952,7 @@ extern "C" im_status im_spread_mc(im_graph* g, const int32_t* seeds, int32_t k, 
         a.words = words;
         a.vis = vis.as<uint32_t>();
         a.gen = gen.as<int32_t>();
+        a.err = reinterpret_cast<uint32_t*>(acc.as<unsigned long long>() + 2);
         a.f_next = F[0].as<uint32_t>();
         a.q_out = Q[0].as<QEntry>();
         a.ctr_out = cp;
@@ -1983,11 +1985,12 @@ extern "C" im_status im_spread_mc(im_graph* g, const int32_t* seeds, int32_t k, 
         if (e == cudaSuccess) e = launch_mc_reduce(reach.as<unsigned long long>(), valid, acc.as<unsigned long long>(), st);
         if (e != cudaSuccess) break;
     }
-    unsigned long long h[2] = {0, 0};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h, acc.p, 16, cudaMemcpyDeviceToHost, st);
+    unsigned long long h[3] = {0, 0, 0};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, acc.p, 24, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     release();
     if (e != cudaSuccess) return cuda_fail(c, e, "spread");
+    if (h[2]) return fail(c, IM_E_STATE, "device index out of bounds (bounds-checked build)");
     const double mean = (double)h[0] / (double)R;
     const long double var = ((long double)h[1] - (long double)h[0] * (long double)h[0] / (long double)R) /
                             (long double)(R - 1);

@@ -375,7 +375,7 @@ __device__ __forceinline__ void list_word(const LevelArgs& a, uint32_t word) {
     }
     if (r == 0) base = atomicAdd(a.awl_count, k);
     base = grp.shfl(base, 0);
-    a.awl[base + r] = word;
+    a.awl[chk((int64_t)(base + r), (int64_t)a.vq_cap * a.words, a.err)] = word;
 }
 
 // Affected-set search (incremental rebuild): marks the simulations of
@@ -1560,7 +1560,8 @@ __device__ __forceinline__ void words_flush(const LevelArgs& a, unsigned int* hd
         at = atomicAdd(a.awl_count, n);
     }
     __syncthreads();
-    for (unsigned i = threadIdx.x; i < n; i += blockDim.x) a.awl[at + i] = hdr[4 + i];
+    for (unsigned i = threadIdx.x; i < n; i += blockDim.x)
+        a.awl[chk((int64_t)(at + i), (int64_t)a.vq_cap * a.words, a.err)] = hdr[4 + i];
 }
 
 // One level per launch (used when the host traces every level).
@@ -2030,7 +2031,8 @@ __global__ void __launch_bounds__(kFBlock) k_bucket_place(GraphDev g, const uint
                                                           const uint32_t* __restrict__ lcm_hi, int J,
                                                           uint32_t* __restrict__ cursor,
                                                           int32_t* __restrict__ other_out,
-                                                          uint16_t* __restrict__ mask_out) {
+                                                          uint16_t* __restrict__ mask_out, int64_t entries,
+                                                          uint32_t* err) {
     __shared__ __align__(16) uint32_t sX[kMaxJ];
     __shared__ uint32_t sBits[kFBlock / 32][64];  // transposed masks of the step
     extern __shared__ uint32_t sBase[];           // [warp][row of the step][chunk]: the reserved place
@@ -2111,7 +2113,7 @@ __global__ void __launch_bounds__(kFBlock) k_bucket_place(GraphDev g, const uint
             const unsigned b_i = __shfl_sync(0xFFFFFFFFu, before, i);
             if (k < total) {
                 const int c = nth_chunk(lo_i, hi_i, k - ex_i);
-                const uint32_t pos = base[r_i * C + c] + (uint32_t)__popc(bits[c] & b_i);
+                const uint32_t pos = chk(base[r_i * C + c] + (uint32_t)__popc(bits[c] & b_i), entries, err);
                 other_out[pos] = o_i;
                 mask_out[pos] = (uint16_t)live16(sX, c, h_i, t_i);
             }
@@ -2205,16 +2207,17 @@ static cudaError_t live_chunks_mode(int kind, const GraphDev& g, const uint32_t*
 
 template <int MODE>
 static cudaError_t place_mode(int kind, const GraphDev& g, const uint32_t* X, const uint32_t* lo, const uint32_t* hi,
-                              int J, uint32_t* cursor, int32_t* other, uint16_t* mask, cudaStream_t st) {
+                              int J, uint32_t* cursor, int32_t* other, uint16_t* mask, int64_t entries, uint32_t* err,
+                              cudaStream_t st) {
     const int C = J >> 4, block = place_block(C);
     const size_t shared = (size_t)(block / 32) * 32 * C * sizeof(uint32_t);
     const int64_t want = ((g.m + 31) / 32 + block / 32 - 1) / (block / 32);
     const int grid = (int)max((int64_t)1, min(want, (int64_t)152 * 8));
     switch (kind) {
-        case kUniform: k_bucket_place<kUniform, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask); break;
-        case kWC: k_bucket_place<kWC, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask); break;
-        case kTrivalency: k_bucket_place<kTrivalency, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask); break;
-        default: k_bucket_place<kExplicit, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask); break;
+        case kUniform: k_bucket_place<kUniform, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask, entries, err); break;
+        case kWC: k_bucket_place<kWC, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask, entries, err); break;
+        case kTrivalency: k_bucket_place<kTrivalency, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask, entries, err); break;
+        default: k_bucket_place<kExplicit, MODE><<<grid, block, shared, st>>>(g, X, lo, hi, J, cursor, other, mask, entries, err); break;
     }
     return cudaGetLastError();
 }
@@ -2258,11 +2261,12 @@ __global__ void __launch_bounds__(kFBlock) k_count_nonzero(const uint32_t* __res
 
 cudaError_t launch_buckets(int pass, int kind, int mode, const GraphDev& g, const uint32_t* X,
                            const uint32_t* lcm_lo, const uint32_t* lcm_hi, int J, uint32_t* cnt_or_end,
-                           unsigned long long* nonempty, int32_t* other, uint16_t* mask, cudaStream_t st) {
+                           unsigned long long* nonempty, int32_t* other, uint16_t* mask, int64_t entries,
+                           uint32_t* err, cudaStream_t st) {
     if (g.m == 0) return cudaSuccess;
     if (pass != 0)
-        return mode == kPush ? place_mode<kPush>(kind, g, X, lcm_lo, lcm_hi, J, cnt_or_end, other, mask, st)
-                             : place_mode<kCover>(kind, g, X, lcm_lo, lcm_hi, J, cnt_or_end, other, mask, st);
+        return mode == kPush ? place_mode<kPush>(kind, g, X, lcm_lo, lcm_hi, J, cnt_or_end, other, mask, entries, err, st)
+                             : place_mode<kCover>(kind, g, X, lcm_lo, lcm_hi, J, cnt_or_end, other, mask, entries, err, st);
     const int64_t want = ((g.m + 31) / 32 + kFBlock / 32 - 1) / (kFBlock / 32);
     const int grid = (int)max((int64_t)1, min(want, (int64_t)152 * 8));
     if (mode == kPush) k_bucket_count<kPush><<<grid, kFBlock, 0, st>>>(g, lcm_lo, lcm_hi, J >> 4, cnt_or_end);

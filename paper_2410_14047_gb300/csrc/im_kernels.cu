@@ -1139,7 +1139,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_mc_level(GraphDev g, McArgs a) {
         if (want) {
             QEntry x;
             x.v = o; x.rp = rp; x.off = (int32_t)(qb & kEdgeMask) + (incl - d); x.aux = 0;
-            a.q_out[(int32_t)(qb >> kCountShift) + __popc(wm & ((1u << lane) - 1u))] = x;
+            a.q_out[chk((int32_t)(qb >> kCountShift) + __popc(wm & ((1u << lane) - 1u)), a.n, a.err)] = x;
         }
     };
     // collects the lanes' hits (edge target o, simulation r), applying 32 at a time

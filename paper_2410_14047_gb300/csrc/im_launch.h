@@ -293,10 +293,11 @@ cudaError_t launch_live_chunks(int kind, int mode, const GraphDev& g, const uint
 // masks (lcm_hi: chunks 32 and up, J > 512).  Pass 0 counts bucket sizes
 // into cnt[n * J/16] (zeroed by the caller) and non-empty buckets into
 // *nonempty; after an exclusive scan of cnt into end[] (end[nb] = total),
-// pass 1 fills other / mask and leaves end[b] = end of bucket b.
+// pass 1 fills other / mask (`entries` of them) and leaves end[b] = end of bucket b.
 cudaError_t launch_buckets(int pass, int kind, int mode, const GraphDev& g, const uint32_t* X,
                            const uint32_t* lcm_lo, const uint32_t* lcm_hi, int J, uint32_t* cnt_or_end,
-                           unsigned long long* nonempty, int32_t* other, uint16_t* mask, cudaStream_t st);
+                           unsigned long long* nonempty, int32_t* other, uint16_t* mask, int64_t entries,
+                           uint32_t* err, cudaStream_t st);
 // Lazy pick: refreshes S_v of every unpicked v whose stored (lb[v], v) is
 // below (S_cand, cand) with S_cand fresh, then takes the least stored pair.
 cudaError_t launch_pick_lazy(const PickArgs& a, cudaStream_t st);
@@ -366,6 +367,7 @@ struct McArgs {
     unsigned long long* ctr_out;
     int32_t* gen;
     int32_t gen_next;
+    uint32_t* err;  // raised by the bounds-checked build only
 };
 int mc_grid();
 cudaError_t launch_mc_level(int kind, const GraphDev& g, const McArgs& a, int grid,
