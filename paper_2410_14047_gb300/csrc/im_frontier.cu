@@ -36,10 +36,7 @@ constexpr int kFBlock = 256;
 using StatT = uint32_t;
 // resident blocks per SM the frontier kernels are compiled for (register cap);
 // the work is latency-bound, so more resident warps hide more of it
-#ifndef IM_PHASE_BLOCK
-#define IM_PHASE_BLOCK 512
-#endif
-constexpr int kPBlock = IM_PHASE_BLOCK;  // threads of a phase kernel's block (two blocks an SM)
+constexpr int kPBlock = 512;  // threads of a phase kernel's block (two blocks an SM)
 constexpr int kPhaseMinBlocks = 1024 / kPBlock;
 constexpr int kLevelMinBlocks = 4;
 
