@@ -11,7 +11,8 @@ import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-def test_callers_at_the_same_time_give_what_each_gives_alone():
+@pytest.mark.parametrize("slots", [(3, 5), (40, 2)], ids=["few", "many"])
+def test_callers_at_the_same_time_give_what_each_gives_alone(slots):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -48,7 +49,7 @@ def test_callers_at_the_same_time_give_what_each_gives_alone():
     B = im.im_batch_load(ctx, graphs, [0.1] * 6)
     alone = {"select": select(G), "steps": steps(G), "batch": batch(B)}
 
-    servers = [im.Server(0, slots=3), im.Server(0, slots=5)]
+    servers = [im.Server(0, slots=k) for k in slots]
     for s in servers:
         s.add_graph(G)
     own = {"select": [], "steps": [], "batch": []}
@@ -63,13 +64,13 @@ def test_callers_at_the_same_time_give_what_each_gives_alone():
     threads = [threading.Thread(target=caller, args=(k,)) for k in own]
     for t in threads:
         t.start()
-    tickets = [[s.submit(**q) for q in kinds * 3] for s in servers]
+    tickets = [[s.submit(**q) for q in kinds * 10] for s in servers]
     results = [[s.wait(k) for k in ts] for s, ts in zip(servers, tickets)]
     for t in threads:
         t.join()
     for rs in results:
-        assert len(rs) == 3 * len(plain)
-        for r, p in zip(rs, plain * 3):
+        assert len(rs) == 10 * len(plain)
+        for r, p in zip(rs, plain * 10):
             assert r["status"] == 0, r["error"]
             assert r["seeds"].tolist() == p["seeds"].tolist()
             assert np.array_equal(r["score"], p["score"])
