@@ -135,12 +135,14 @@ typedef struct {
 /* Schedule knobs of the frontier kernels (chosen by the autotuner; results
  * do not depend on them).  heavy_indeg: in-degree above which a vertex whose
  * in-edges share one threshold below 2^26 (weighted cascade, small uniform p)
- * is pushed by per-simulation hash search instead of an in-edge scan;
+ * is pushed by per-simulation hash search instead of an in-edge scan, as long
+ * as fewer than three of its in-edges agree with a simulation above the
+ * threshold's top bit on average (always so for weighted cascade);
  * light_batches: 32-edge batches a warp claims at once; grid_blocks: blocks
  * per frontier launch (0 = SM count x occupancy); check_every: frontier
  * launches between the host's first two emptiness checks (then doubling to 8);
  * persistent: 1 = all levels of a phase in one cooperative launch with grid
- * barriers between levels (per-level launches when tracing); dense_div: a
+ * barriers between levels, 0 = a launch a level; dense_div: a
  * propagation level whose frontier exceeds (vertices with in-edges) /
  * dense_div walks every such vertex in vertex order (0 = never; the first
  * level of a build always does when dense_div > 0); lazy_pick: 1 = in

@@ -15,14 +15,15 @@
 // the sorted X), then the batch's 16-simulation chunks that hold a changed
 // simulation are dealt to the lanes; a chunk moves 16 register bytes with one
 // 16-byte load and merges them with a byte-wise max (Eq. sketch-merge) through
-// CAS on 4-byte words, only where a register improves.
+// a 16-byte CAS, only where a register improves.
 //
 // Heavy vertex v (weighted-cascade or uniform model, threshold below 2^26, few
-// in-edges per candidate interval: is_heavy): every in-edge of v has the same threshold, and in-rows are sorted by edge
-// hash, so the in-edges live in simulation j are inside one hash interval
-// (the edge hash must agree with X_j above the threshold's top bit).  Each
-// changed simulation costs two binary searches in v's row plus the live
-// candidates, instead of a scan of all in-edges.
+// in-edges per candidate interval: is_heavy): every in-edge of v has the same
+// threshold, and in-rows are sorted by edge hash, so the in-edges live in
+// simulation j are inside one hash interval (the edge hash must agree with X_j
+// above the threshold's top bit).  Each changed simulation costs two binary
+// searches in v's row plus the live candidates, instead of a scan of all
+// in-edges.
 #include <cooperative_groups.h>
 
 #include "im_host.h"
@@ -84,7 +85,8 @@ __device__ __forceinline__ int32_t first_window(const QEntry* __restrict__ q, in
 // memory and moves them to the queue together at the level's end (block_flush):
 // one reservation a block and level, not one a warp and batch on a single
 // counter, and no warp waits for a reservation's reply (R-MAT scale 20, weighted
-// cascade, J = 256, K = 50: 102.5 -> 97.2 ms; 64 batched graphs: 222 -> 208 ms).
+// cascade, J = 256, K = 50: 102.5 -> 97.2 ms; 64 batched graphs: 1.068 times as
+// fast).
 // Layout: entries taken, the first place that did not fit, then the
 // entries (off: the entry's edges).  A warp that finds the buffer full queues
 // its entries itself.
@@ -158,9 +160,10 @@ __device__ __forceinline__ uint32_t bytes_to_bits(uint32_t d) {
 
 // Where a vertex whose registers changed goes for the next propagation
 // level: the heavy queue (one warp searches the in-row per changed simulation)
-// when it is an in-degree hub whose in-edges share one small threshold and at
-// most kHeavyCand in-edges agree with a simulation above the threshold's top
-// bit on average, else the light queue (its in-edges are scanned).  A search
+// when it is an in-degree hub whose in-edges share one small threshold and
+// fewer than kHeavyCand + 1 in-edges agree with a simulation above the
+// threshold's top bit on average (the shift rounds down), else the light queue
+// (its in-edges are scanned).  A search
 // pushes one register at a time along each candidate, in one warp's chain of
 // dependent loads and CAS; a scan moves 16 registers an item and spreads over
 // warps, so the search only wins while a simulation has about one candidate
@@ -473,7 +476,7 @@ __device__ __forceinline__ void newly_visited(const LevelArgs& a, int32_t o, uin
     if (a.gcount) {
         // a batch counts per graph: the lanes of a graph together (the lanes of
         // a 32-edge batch are mostly one graph's, and single adds queued up on
-        // a few counters: 64 graphs took 207.5 ms, and 188.7 ms this way)
+        // a few counters: 64 graphs are 1.099 times as fast this way)
         const int32_t g = __ldg(a.gid + o);
         const unsigned peers = __match_any_sync(__activemask(), g);
         const unsigned sum = __reduce_add_sync(peers, k);
